@@ -54,7 +54,7 @@ void vv10_ctx::release_all() {
     batch_release();
     DevBuf* bufs[] = {&prep_hist, &prep_offs, &prep_bbox, &prep_small, &orig, &seg, &atom_k,
                       &soa, &r64a, &r64b, &r32a, &r32b, &r32p, &sumE, &sumU, &sumW, &sumA, &sumB,
-                      &sumC, &part, &eblk, &scal, &tu, &ty, &trt, &tgt, &hacc, &gk,
+                      &sumC, &part, &symw, &eblk, &scal, &tu, &ty, &trt, &tgt, &hacc, &gk,
                       &tc_uh, &tc_ul, &tc_yh, &tc_yl, &tc16_bh, &tc16_bl, &tc16_small, &o64_sl, &o64_small, &o64_rec, &hvp_fr, &hvp_fg, &nhess, &chpart, &wdir, &wsplit, &ehalf, &aophik, &aoz, &aom, &aogw, &aofa, &ngpart, &dev_err};
     for (DevBuf* b : bufs) {
         if (b->p) cudaFree(b->p);
@@ -401,6 +401,19 @@ vv10_status vv10_ctx::require_prepared() {
 vv10_status vv10_ctx::run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_split_out) {
     if (autotune & VV10_TUNE_PAIRSUMS) VV10_TRY(tune_pairsum(mode, fp64, st, false));
     const int nq = pair_mode_nq(mode);
+    const int phase = (mode == MODE_EUW || mode == MODE_EUWABC || mode == MODE_EUWABCG) ? PH_PAIR_EUW
+                      : (mode == MODE_ABC ? PH_PAIR_ABC : PH_PAIR_GRAD);
+    if (!debug_stall && pairsum_sym(mode, fp64)) {
+        VV10_TRY(ensure(part, sizeof(double) * nq * static_cast<size_t>(P.nk_pad), "pair sums"));
+        int n_launch = 0;
+        VV10_TRY(ensure(symw, pairsum_sym_work(P.nk_pad, mode, fp64, n_sm, &n_launch), "pair-sum partials"));
+        PhaseScope ph(this, phase, st, n_launch);
+        launches[PH_EP_EPILOGUE] += n_launch;  // the reductions of their partial sums
+        VV10_CUDA(this, launch_pairsum_sym(P, mode, fp64, n_sm, symw.p, static_cast<double*>(part.p), st),
+                  "pair-sum kernel");
+        *n_split_out = 1;
+        return VV10_OK;
+    }
     PairLaunch cfg;
     const TileChoice tc = tiles_for(mode, fp64);
     cfg.rows_per_thread = tc.rows_per_thread;
@@ -413,15 +426,23 @@ vv10_status vv10_ctx::run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_s
     VV10_TRY(ensure(part, sizeof(double) * nq * static_cast<size_t>(ns) * (P.nk_pad > 0 ? P.nk_pad : 1),
                     "pair-sum partials"));
     {
-        PhaseScope ph(this, (mode == MODE_EUW || mode == MODE_EUWABC || mode == MODE_EUWABCG) ? PH_PAIR_EUW
-                            : (mode == MODE_ABC ? PH_PAIR_ABC : PH_PAIR_GRAD),
-                      st, 1);
+        PhaseScope ph(this, phase, st, 1);
         VV10_CUDA(this, launch_pairsum(P, mode, fp64, cfg, static_cast<double*>(part.p),
                                        static_cast<int*>(dev_err.p), st),
                   "pair-sum kernel");
     }
     *n_split_out = ns;
     return VV10_OK;
+}
+
+// Whether a mode's sums run over unordered pairs: at the sizes where that is faster, unless
+// vv10_set_tiles fixed a shape of the row-by-row kernel.
+bool vv10_ctx::pairsum_sym(int mode, bool fp64) const {
+    const TileOverride& o = overrides[mode + kPairModes * (fp64 ? 1 : 0)];
+    const TileOverride& e = overrides[MODE_EUW + kPairModes * (fp64 ? 1 : 0)];
+    const bool fused = (mode == MODE_EUWABC || mode == MODE_EUWABCG);
+    const TileOverride* use = o.active ? &o : ((fused && e.active) ? &e : nullptr);
+    return !(use && use->manual) && pairsum_sym_applies(P.nk, fp64);
 }
 
 // Tiles of a pair-sum mode: its own override (fixed or tuned), else (fused mode) the

@@ -127,11 +127,15 @@ vv10_status vv10_ctx::tune_pairsum(int mode, bool fp64, cudaStream_t st, bool fo
         o = TileOverride{true, false, mode, fp64, rpt, ns, nb};
         return VV10_OK;
     }
+    float best = 3.0e38f;
+    int best_r = fp64 ? 1 : 2, best_s = 0;
+    if (pairsum_sym(mode, fp64)) {  // no shape to choose: the unordered-pair kernel runs
+        o = TileOverride{true, false, mode, fp64, best_r, pairsum_default_split(P, mode, fp64, best_r, n_sm), nb};
+        return VV10_OK;
+    }
     if (stream_capturing(st)) return VV10_OK;
     QuietScope quiet(this);
     const std::vector<int> rpts = fp64 ? std::vector<int>{1, 2} : std::vector<int>{1, 2, 4};
-    float best = 3.0e38f;
-    int best_r = fp64 ? 1 : 2, best_s = 0;
     for (int r : rpts) {
         const int d = pairsum_default_split(P, mode, fp64, r, n_sm);
         std::vector<int> splits = {d};

@@ -155,6 +155,15 @@ cudaError_t launch_pairsum(const PointsDev& p, int mode, bool fp64, const PairLa
                            double* part, int* err, cudaStream_t st);
 int pairsum_default_split(const PointsDev& p, int mode, bool fp64, int rows_per_thread, int n_sm);
 
+// The same sums over unordered pairs (pairsum_sym.cu): total[nq][nk_pad] FP64, one split; `work`
+// holds pairsum_sym_work() bytes (n_launch: launches of the pair kernel, each followed
+// by one of its reduction).  pairsum_sym_applies: the
+// sizes at which it is the faster one.
+bool pairsum_sym_applies(int64_t nk, bool fp64);
+size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, int* n_launch);
+cudaError_t launch_pairsum_sym(const PointsDev& p, int mode, bool fp64, int n_sm, void* work,
+                               double* total, cudaStream_t st);
+
 // Batched pair sums (batch.cu): one persistent launch over a task table with an atomic
 // work counter.  PairMol describes one molecule's records and partial buffer
 // part[nq][n_split][nk_pad]; PairTask one (molecule, row tile, j-split) unit.

@@ -138,6 +138,7 @@ struct vv10_ctx {
 
     // pair-sum partials and energy reduction scratch
     vv10::DevBuf part, eblk, scal;
+    vv10::DevBuf symw;  // row totals and column sums of the unordered-pair kernel
 
     // Hessian scratch
     vv10::DevBuf tu, ty, trt, tgt, hacc;
@@ -211,6 +212,7 @@ struct vv10_ctx {
     vv10_status require_prepared();
     vv10::PointsDev points() const;
     vv10::TileChoice tiles_for(int mode, bool fp64) const;
+    bool pairsum_sym(int mode, bool fp64) const;
     vv10_status run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_split_out);
     // autotuner (autotune.cu)
     vv10_status tune_pairsum(int mode, bool fp64, cudaStream_t st, bool force);
