@@ -26,14 +26,23 @@
 // about the same time (they stay in L2 at any N), and every output row is updated by one
 // CTA only, in a fixed order (no atomics).
 //
-// 16 warps per CTA (4 per TMEM lane quadrant, 8 j each), every one of which, per stage:
-// evaluates its part of the two (or four) kernel tiles, exchanges the row maxima of the
-// stage with the quadrant's other warps through shared memory, scales, splits and stores
-// its operand columns into TMEM, then drains the previous stage's accumulator.  Two single
-// threads carry the other roles inside that loop, so that each warp keeps 128 registers
-// (four warps per SM sub-partition): lane 0 of warp 0 issues the stage's MMAs once every
-// warp's operands are in place, lane 0 of warp 1 keeps the ring of copies (j records by
-// 1-D bulk copy, the hi and lo trial tiles by 2-D tensor copies) kF16Ring - 1 stages ahead.
+// Roles (20 warps).  Eight warps generate: evaluate the kernel tiles of a stage, find the row
+// maximum, scale, split and store the operands into TMEM.  With one output kind (Ppad > 64) the two
+// generating warpgroups take alternate stages, each thread all 32 j of its row: the maximum needs
+// no exchange and the warps of a scheduler run out of step, one in its FMA-bound tile arithmetic
+// while the other splits and stores; the tiles of 12 of the 32 j wait for the maximum in shared
+// memory, the rest in registers.  With both kinds a thread takes 16 j and the two warps of a row
+// exchange maxima.  Eight warps drain the accumulators into FP32 registers (half of the columns
+// each).  One thread issues the MMAs and one the copies (j records by 1-D bulk copy, the hi and lo
+// trial tiles by 2-D tensor copies).  The issuing thread is held by the tensor pipe's short queue
+// for most of a stage's MMAs (960 of 1,250 cycles at Ppad = 192); when it was a lane of a generating
+// warp, as in the earlier 16-warp form, all the others waited for that warp.
+//
+// What bounds it: per 128 x 32 stage 1,250 cycles of MMA at Ppad = 192 (2,000 for both kinds at 64)
+// and about 1,300 of FMA pipe; the stage takes about 3,400 (3,700), the rest being dependent-issue
+// latency of two generating warps a scheduler.  Contraction alone, milliseconds, before and now:
+// 80,889 points P = 180 47.4, 39.9; 39,696 P = 128 12.6, 10.1; 32,598 P = 72 8.1, 6.5; 29,778
+// P = 54 4.8, 3.7.
 // Every wait is bounded (kSpinCycles); a wait that gives up sets the TIMEOUT bit and an
 // abort flag that ends the other waits.
 #include <cstring>
@@ -48,10 +57,18 @@
 namespace vv10 {
 
 constexpr int kF16Kj = 32;                      // j per stage
-constexpr int kF16Warps = 16;                   // every warp generates and drains
-constexpr int kF16ProducerWarp = 1;             // lane 0 also issues the copies
-constexpr int kF16MmaWarp = 0;                  // lane 0 also issues the MMAs; owns TMEM
-constexpr int kF16Threads = kF16Warps * 32;
+constexpr int kF16GenWarps = 8;                 // warpgroups 0, 1: generate the operands
+constexpr int kF16DrainWarps = 8;               // warpgroups 2, 3: drain the accumulators
+constexpr int kF16MmaWarp = 16;                 // lane 0 issues the MMAs; owns TMEM
+constexpr int kF16ProducerWarp = 17;            // lane 0 issues the copies
+constexpr int kF16Threads = 20 * 32;            // warpgroup 4: the two roles and two idle warps
+// Registers: 20 warps are launched with 96 a thread (five warps a scheduler); the warpgroups then
+// take what they need, 8 gen + 8 drain + 4 role = 20 x 96.
+constexpr int kF16RoleRegs = 32;
+constexpr int kF16Park = 6;                     // NK = 1: pairs of j whose tiles wait in shared memory
+template <int PPAD> constexpr int f16_drain_regs() { return PPAD > 128 ? 120 : 104; }
+template <int PPAD> constexpr int f16_gen_regs() { return 224 - f16_drain_regs<PPAD>(); }
+static_assert(8 * 224 + 4 * kF16RoleRegs <= 20 * 96, "register shares within the launch's");
 constexpr int kF16Ring = 4;                     // stages of trial tiles in flight
 constexpr int kF16MaxPpad = 192;
 constexpr uint32_t kF16TmemCols = 512;
@@ -61,8 +78,9 @@ struct F16Layout {
     uint32_t tile_bytes;  // one Ppad x 64-half trial tile (128-byte rows: 16 u, 16 y, 16 u, 16 y)
     uint32_t slot_bytes;  // hi and lo tiles of one stage
     uint32_t rec_off;     // j records, 1024 B per stage
-    uint32_t xm_off;      // row-maximum exchange [2][4 quads][NK][32 lanes][4 parts] floats
-    uint32_t prod_off;    // the producer thread's state
+    uint32_t xm_off;      // NK = 2: row-maximum exchange [2][4 quads][NK][32 lanes][2 parts] floats
+    uint32_t stg_off;     // NK = 1: parked tiles [8 warps][kF16Park][2][32 lanes] float2
+    uint32_t isc_off;     // inverse row factors [kF16Ring][NK][128 rows] floats
     uint32_t bar_off;
     uint32_t total;
 };
@@ -72,8 +90,9 @@ __host__ __device__ inline F16Layout f16_layout(int ppad, int nk) {
     L.slot_bytes = 2u * L.tile_bytes;
     L.rec_off = kF16Ring * L.slot_bytes;
     L.xm_off = L.rec_off + kF16Ring * 1024u;
-    L.prod_off = L.xm_off + 2u * 4u * static_cast<uint32_t>(nk) * 32u * 16u;
-    L.bar_off = L.prod_off + 128u;
+    L.stg_off = L.xm_off + (nk == 2 ? 2u * 4u * 2u * 32u * 8u : 0u);
+    L.isc_off = L.stg_off + (nk == 2 ? 0u : 8u * kF16Park * 512u);
+    L.bar_off = L.isc_off + kF16Ring * static_cast<uint32_t>(nk) * 512u;
     L.total = L.bar_off + 512u + 1024u;  // barriers + slack for the 1024-B alignment
     return L;
 }
@@ -134,7 +153,7 @@ __device__ __forceinline__ bool f16_wait(uint64_t* bar, uint32_t parity, int* er
 //   T3c = rp (nA_j M + L + G_i)                                   = T3 / (+3/2)
 //   T4c = rp R^2 M                                                = T4 / (-3/2)
 // (the factors -3/2, +3/2 travel with the trials).  NK = 2: t = {T1c, T2c, T3c, T4c};
-// NK = 1: the two tiles of output `kind`.
+// NK = 1: the two tiles of output `kind`; `fuse_j`: how its L + G_j is rounded (below).
 struct RowF {
     float x, y, z, om, ka, np, nq;  // row i values; np = -p_i, nq = -q_i
 };
@@ -143,7 +162,7 @@ __device__ __forceinline__ float2 f16_lo2(float4 v) { return make_float2(v.x, v.
 __device__ __forceinline__ float2 f16_hi2(float4 v) { return make_float2(v.z, v.w); }
 
 template <int NK>
-__device__ __forceinline__ void f16_tiles2(int kind, const RowF& r, const float4 v0,
+__device__ __forceinline__ void f16_tiles2(int kind, bool fuse_j, const RowF& r, const float4 v0,
                                            const float4 v1, const float4 v2, const float4 v3,
                                            float2 (&t)[2 * NK]) {
     const float2 one = make_float2(1.0f, 1.0f), two = make_float2(2.0f, 2.0f);
@@ -163,13 +182,18 @@ __device__ __forceinline__ void f16_tiles2(int kind, const RowF& r, const float4
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv.y) : "f"(den.y));
     const float2 L = __fmul2_rn(ggp, inv);
     const float2 sinv = __fmul2_rn(s, inv);  // 1/(g g')
-    const float2 Gi = __fmul2_rn(gp, sinv);
-    const float2 Gj = __fmul2_rn(g, sinv);
     const float2 M = __fmul2_rn(two, __ffma2_rn(L, L, sinv));
     const float2 nAi = __ffma2_rn(f16_dup(r.nq), r2, f16_dup(r.np));
     const float2 nAj = __ffma2_rn(f16_lo2(v3), r2, f16_hi2(v2));
     const float2 rp = __fmul2_rn(r2, inv);
-    const float2 LGi = __fadd2_rn(L, Gi), LGj = __fadd2_rn(L, Gj);
+    // L + G_i and L + G_j, the product in G fused into the sum.  The assembler fuses a packed
+    // product and sum on its own where it likes, so both forms are written out; with one output
+    // kind, three of four pairs take L + G_j unfused, the roundings this contraction has had
+    // (fused everywhere the results move by 3e-9, a fortieth of their error).
+    const float2 LGi = __ffma2_rn(gp, sinv, L);
+    const float2 Gj = __fmul2_rn(g, sinv);
+    const float2 LGj = NK == 2 || fuse_j ? __ffma2_rn(g, sinv, L)
+                                         : make_float2(__fadd_rn(L.x, Gj.x), __fadd_rn(L.y, Gj.y));
     if (NK == 2 || kind == 0) {
         float2 br = __ffma2_rn(nAi, LGi, one);
         br = __ffma2_rn(nAj, LGj, br);
@@ -225,7 +249,7 @@ __device__ __forceinline__ uint32_t f16_acol(int b) {
 // of truth: the other roles follow it).
 enum : int32_t { F16_FIRST = 1, F16_LAST = 2, F16_END = 4 };
 struct F16Meta {
-    int32_t mol, row_tile, kind, flags;
+    int32_t mol, row_tile, kind, flags;  // flags: F16_* and, from bit 3, the unit's number
 };
 
 // The producer's position in the walk.  Single system: (j chunk c, unit u, stage s), units
@@ -237,14 +261,6 @@ struct F16Cursor {
     int32_t mol, row_tile, kind;
     bool done;
 };
-// The producer thread's state (shared memory).
-struct F16Prod {
-    F16Cursor k;
-    int64_t issued;
-    int32_t slot, mol;
-    uint32_t ph, end;
-};
-
 // Batch: the next task from the CTAs' shared counter (false once every task is taken).
 __device__ __forceinline__ bool f16_next_task(F16Cursor& k, const F16Args& a) {
     const int64_t q = atomicAdd(a.counter, 1);
@@ -298,11 +314,11 @@ __device__ __forceinline__ void f16_cursor_next(F16Cursor& k, const F16Args& a) 
     k.s = k.s0;
 }
 
-template <int PQ, int NK>  // PQ accumulator columns per thread and kind (= Ppad / 4)
+template <int PPAD, int NK>
 __global__ void __launch_bounds__(kF16Threads, 1)
 k_hess_f16(const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CUtensorMap tm_bl,
            F16Args args) {
-    constexpr int PPAD = 4 * PQ;
+    constexpr int GP = NK;  // generating warps per stage and quad
     static_assert(NK == 1 || PPAD <= 64, "two kinds per tile need Ppad <= 64");
     static_assert(NK == 2 || 2 * PPAD + 128 <= static_cast<int>(kF16TmemCols), "TMEM columns");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -310,32 +326,32 @@ k_hess_f16(const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CU
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const F16Layout L = f16_layout(PPAD, NK);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bar_off);
-    uint64_t* b_full = bars;                          // [kF16Ring]
-    uint64_t* b_empty = bars + kF16Ring;              // [kF16Ring]
-    uint64_t* a_full = bars + 2 * kF16Ring;           // [2]
+    uint64_t* b_full = bars;                          // [kF16Ring] a stage's copies and metadata
+    uint64_t* b_empty = bars + kF16Ring;              // [kF16Ring] every drain warp has its MMAs behind it
+    uint64_t* a_full = bars + 2 * kF16Ring;           // [2] operands in TMEM
     uint64_t* mma_done = bars + 2 * kF16Ring + 2;     // [2]
-    uint64_t* xbar = bars + 2 * kF16Ring + 4;         // [2 slots][4 quads]
-    uint64_t* fin = bars + 2 * kF16Ring + 12;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kF16Ring + 13);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kF16Ring + 14);
-    F16Meta* meta = reinterpret_cast<F16Meta*>(bars + 2 * kF16Ring + 16);  // [kF16Ring]
-    float* xm = reinterpret_cast<float*>(smem + L.xm_off);
+    uint64_t* acc_free = bars + 2 * kF16Ring + 4;     // [2] accumulator drained
+    uint64_t* xbar = bars + 2 * kF16Ring + 6;         // [2][4 quads] NK = 2: both row maxima stored
+    uint64_t* fin = bars + 2 * kF16Ring + 14;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kF16Ring + 15);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kF16Ring + 16);
+    F16Meta* meta = reinterpret_cast<F16Meta*>(bars + 2 * kF16Ring + 18);  // [kF16Ring]
+    float* iscs = reinterpret_cast<float*>(smem + L.isc_off);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int quad = warp & 3, part = warp >> 2;
-    const bool is_producer = (warp == kF16ProducerWarp && lane == 0);
-    const bool is_mma = (warp == kF16MmaWarp && lane == 0);
+    const int quad = warp & 3;  // TMEM lanes 32 quad .. (a warp reaches those of its index mod 4)
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < kF16Ring; ++b) {
             mbar_init(&b_full[b], 1);
-            mbar_init(&b_empty[b], kF16Warps);
+            mbar_init(&b_empty[b], kF16DrainWarps);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&a_full[b], kF16Warps);
+            mbar_init(&a_full[b], 4 * GP);
             mbar_init(&mma_done[b], 1);
+            mbar_init(&acc_free[b], kF16DrainWarps);
         }
-        for (int b = 0; b < 8; ++b) mbar_init(&xbar[b], 4);  // one arrival per warp of a quad
+        for (int b = 0; b < 8; ++b) mbar_init(&xbar[b], 2);
         mbar_init(fin, 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -345,224 +361,255 @@ k_hess_f16(const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CU
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = *tmem_slot;
-
-    // ---------------------------------------------------------------- producer (one thread)
-    // keeps the ring kF16Ring - 1 stages ahead of the walk; every stage's copies complete on
-    // its b_full barrier together with the producer's arrival, which releases the metadata.
-    // Its state lives in shared memory (only one thread touches it), not in every thread's
-    // registers.
-    F16Prod* pr = reinterpret_cast<F16Prod*>(smem + L.prod_off);
-    bool ok = true;
-    auto produce = [&]() -> bool {
-        F16Prod& P = *pr;
-        if (P.end) return true;
-        if (!f16_wait(&b_empty[P.slot], P.ph ^ 1u, args.err, abort_flag)) return false;
-        if (P.k.done) {  // the end of the walk takes one slot, with no copies
-            meta[P.slot] = F16Meta{0, 0, 0, F16_END};
-            mbar_arrive(&b_full[P.slot]);
-            P.end = 1;
-            return true;
-        }
-        const F16Mol& M = args.mols ? args.mols[P.k.mol] : args.single;
-        const CUtensorMap* mh = &tm_bh;
-        const CUtensorMap* ml = &tm_bl;
-        if (args.mols) {
-            mh = M.maps;
-            ml = M.maps + 1;
-            if (P.k.mol != P.mol) {  // a new molecule's tensor maps
-                P.mol = P.k.mol;
-                tmap_acquire(mh);
-                tmap_acquire(ml);
-                tc::prefetch_tmap(mh);
-                tc::prefetch_tmap(ml);
-            }
-        }
-        const int s = P.k.s;
-        meta[P.slot] = F16Meta{P.k.mol, P.k.row_tile, P.k.kind,
-                               (s == P.k.s0 ? F16_FIRST : 0) | (s == P.k.s1 - 1 ? F16_LAST : 0)};
-        uint8_t* base = smem + P.slot * L.slot_bytes;
-        uint8_t* rec = smem + L.rec_off + P.slot * 1024;
-        mbar_expect_tx(&b_full[P.slot], L.slot_bytes + 1024u);
-        bulk_g2s(rec, M.r32p + 2 * kF16Kj * static_cast<int64_t>(s), 1024u, &b_full[P.slot]);
-        // the chunk's trial tiles are re-read by every unit: keep them in L2 before other lines
-        const uint64_t pol = tc::l2_evict_last();
-        tc::tma_load_2d_hint(base, mh, 64 * s, M.t0, &b_full[P.slot], pol);
-        tc::tma_load_2d_hint(base + L.tile_bytes, ml, 64 * s, M.t0, &b_full[P.slot], pol);
-        ++P.issued;
-        if (++P.slot == kF16Ring) {
-            P.slot = 0;
-            P.ph ^= 1u;
-        }
-        f16_cursor_next<NK>(P.k, args);
-        return true;
-    };
-    if (is_producer) {
-        F16Prod& P = *pr;
-        P.slot = 0;
-        P.ph = 0;
-        P.end = 0;
-        P.mol = -1;
-        P.issued = 0;
-        f16_cursor_init<NK>(P.k, args);
-        if (!args.mols) {
-            tc::prefetch_tmap(&tm_bh);
-            tc::prefetch_tmap(&tm_bl);
-        }
-        for (int k = 0; k < kF16Ring - 1 && ok; ++k) ok = produce();
-        if (!ok) *abort_flag = 1;
-    }
-
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const uint32_t idesc = tc::idesc_f16(128, PPAD);
-    float acc[NK][PQ];
-#pragma unroll
-    for (int k = 0; k < NK; ++k)
-#pragma unroll
-        for (int c = 0; c < PQ; ++c) acc[k][c] = 0.0f;
 
-    // Drain a finished accumulator (every kind of the unit) into the FP32 registers, each
-    // value times the inverse row factor of its stage.
-    auto drain = [&](int db, uint32_t dphase, int kind0, const float (&iscp)[NK]) -> bool {
-        const bool got = f16_wait(&mma_done[db], dphase, args.err, abort_flag);
-        if (!__all_sync(0xffffffffu, got)) return false;  // warp-uniform exit
-        tc::fence_after();
+    // Stage g of the walk: ring slot g mod 4 (pass g / 4), operand and accumulator buffer g mod 2
+    // (use g / 2).
+    if (warp < kF16GenWarps) {
+        // ---------------------------------------------------------------- operand generation
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(f16_gen_regs<PPAD>()));
+        // One output kind: the two warpgroups take alternate stages, a warp all 32 j of its rows
+        // (the row maximum stays in the thread).  Both kinds: each takes 16 j of every stage.
+        constexpr int NH = 16 / GP;  // pairs of j per warp and stage
+        constexpr int NS = GP == 1 ? kF16Park : 0;  // of which parked in shared memory
+        float2* park = reinterpret_cast<float2*>(smem + L.stg_off) + warp * (NS * 64) + lane;
+        const int part = GP == 2 ? warp >> 2 : 0;
+        float* xm = reinterpret_cast<float*>(smem + L.xm_off);
+        RowF rc{0.f, 0.f, 0.f, 1.f, 1.f, 0.f, 0.f};
+        float inv_cy = 1.f;
+        int unit = -1;
+        for (uint32_t g = GP == 2 ? 0 : warp >> 2;; g += 3 - GP) {
+            const int slot = g & 3, ab = g & 1;
+            bool got = f16_wait(&b_full[slot], (g >> 2) & 1u, args.err, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) break;
+            const F16Meta m = meta[slot];
+            if (m.flags & F16_END) break;
+            if ((m.flags >> 3) != unit) {  // a new unit: its rows and molecule
+                unit = m.flags >> 3;
+                const F16Mol& M = args.mols ? args.mols[m.mol] : args.single;
+                const int64_t i = static_cast<int64_t>(m.row_tile) * 128 + quad * 32 + lane;
+                float xi = 0.f, yi = 0.f, zi = 0.f, oi = 1.f, ki = 1.f, pi_ = 0.f, qi = 0.f;
+                if (i < M.nk) {
+                    const float4 a4 = M.r32a[i];
+                    const float4 b4 = M.r32b[i];
+                    xi = a4.x; yi = a4.y; zi = a4.z; oi = b4.x; ki = b4.y; pi_ = b4.z; qi = b4.w;
+                }
+                rc = RowF{xi, yi, zi, oi, ki, -pi_, -qi};
+                inv_cy = M.params[0];
+            }
+            const float4* rec = reinterpret_cast<const float4*>(smem + L.rec_off + slot * 1024) + 4 * NH * part;
+            float2 t[NH - NS][2 * NK];
+            float mx[NK];
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const uint32_t col = tmem + lane_off + f16_dcol<NK, PPAD>(NK == 2 ? k : kind0, db) + part * PQ;
-            constexpr int kChunk = PQ % 16 == 0 ? 16 : 8;
+            for (int k = 0; k < NK; ++k) mx[k] = 0.f;
 #pragma unroll
-            for (int c0 = 0; c0 < PQ; c0 += kChunk) {
-                uint32_t r[kChunk];
+            for (int h = 0; h < NH; ++h) {
+                if (h % 4 == 0) asm volatile("" ::: "memory");  // four chains at a time: registers
+                const float4* v = rec + 4 * h;
+                float2 u[2 * NK];
+                f16_tiles2<NK>(m.kind, h % 4 == 3, rc, v[0], v[1], v[2], v[3], u);
 #pragma unroll
-                for (int c = 0; c < kChunk; c += 8)
-                    tc::ld_x8(col + c0 + c, *reinterpret_cast<uint32_t(*)[8]>(&r[c]));
-                tc::wait_ld();
+                for (int k = 0; k < NK; ++k) {  // the tiles that multiply y carry 1/c_y
+                    u[2 * k + 1] = __fmul2_rn(u[2 * k + 1], make_float2(inv_cy, inv_cy));
+                    mx[k] = fmaxf(mx[k], f16_absmax4(u[2 * k], u[2 * k + 1]));
+                }
 #pragma unroll
-                for (int c = 0; c < kChunk; c += 2) {
-                    const float2 v = __ffma2_rn(make_float2(__uint_as_float(r[c]), __uint_as_float(r[c + 1])),
-                                                make_float2(iscp[k], iscp[k]),
-                                                make_float2(acc[k][c0 + c], acc[k][c0 + c + 1]));
-                    acc[k][c0 + c] = v.x;
-                    acc[k][c0 + c + 1] = v.y;
+                for (int q = 0; q < 2 * NK; ++q) {
+                    if (h < NS) park[(h * 2 + q) * 32] = u[q];
+                    else t[h - NS][q] = u[q];
                 }
             }
-        }
-        tc::fence_before();
-        return true;
-    };
-    // Add the registers into the molecule's FP64 partial output (times 1/s_t; the gamma
-    // accumulator holds -(T3 u + T4 y)) and clear them.
-    auto flush = [&](int mol, int kind0, int64_t i) {
-        const F16Mol& M = args.mols ? args.mols[mol] : args.single;
+            if (GP == 2) {  // the row's largest |T| over the stage: this warp's 16 j and the other's
+                float2* xrow = reinterpret_cast<float2*>(xm) + (static_cast<size_t>((ab * 4 + quad) * NK) * 32 + lane);
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const int kind = NK == 2 ? k : kind0;
+                for (int k = 0; k < NK; ++k) (part ? xrow[k * 32].y : xrow[k * 32].x) = mx[k];
+                __syncwarp();  // the warp's 32 stores are ordered before lane 0's release
+                if (lane == 0) mbar_arrive(&xbar[ab * 4 + quad]);
+                got = f16_wait(&xbar[ab * 4 + quad], (g >> 1) & 1u, args.err, abort_flag);
+                if (!__all_sync(0xffffffffu, got)) break;
 #pragma unroll
-            for (int c = 0; c < PQ; ++c) {
-                const int t = part * PQ + c;
-                if (i < M.nk && t < M.Pn) {
-                    const int64_t tg = static_cast<int64_t>(M.t0) + t;
-                    double* o = M.acc + ((static_cast<int64_t>(kind) * M.acc_P + tg) * M.nk_pad + i);
-                    const double v = static_cast<double>(acc[k][c]) * M.col_isc[tg];
-                    // streaming loads and stores: the partial output must not evict the
-                    // chunk's trial tiles from L2
-                    __stcs(o, __ldcs(o) + ((kind == 0) ? v : -v));
+                for (int k = 0; k < NK; ++k) {
+                    const float2 q = xrow[k * 32];
+                    mx[k] = fmaxf(q.x, q.y);
                 }
-                acc[k][c] = 0.0f;
             }
-        }
-    };
-
-    int slot = 0, ab = 0;
-    uint32_t ph = 0, aph = 0;
-    int pslot = 0, dbuf = 0;
-    uint32_t dph = 0;
-    uint32_t gs = 0;  // stages walked by this CTA (exchange slot and phase)
-    bool mma_any = false;
-    float isc_prev[NK];
+            float sc[NK], isc[NK];
 #pragma unroll
-    for (int k = 0; k < NK; ++k) isc_prev[k] = 1.0f;
-    // the current unit: molecule, output kind, row, row data, 1/c_y
-    int mol = 0, kind0 = 0, until_flush = args.flush;
-    int64_t i = 0;
-    float inv_cy = 1.f;
-    RowF rc{0.f, 0.f, 0.f, 1.f, 1.f, 0.f, 0.f};
-    ok = __all_sync(0xffffffffu, !*abort_flag);
-    while (ok) {
-        // the operand buffer ab is free once the MMAs of the stage two back are done
-        bool got = f16_wait(&b_full[slot], ph, args.err, abort_flag);
-        got = got && f16_wait(&mma_done[ab], aph ^ 1u, args.err, abort_flag);
-        if (!__all_sync(0xffffffffu, got)) break;
-        tc::fence_after();
-        const F16Meta m = meta[slot];
-        if (m.flags & F16_END) break;
-        if (m.flags & F16_FIRST) {  // a new unit: its rows and molecule
-            mol = m.mol;
-            kind0 = NK == 2 ? 0 : m.kind;
-            const F16Mol& M = args.mols ? args.mols[mol] : args.single;
-            i = static_cast<int64_t>(m.row_tile) * 128 + quad * 32 + lane;
-            float xi = 0.f, yi = 0.f, zi = 0.f, oi = 1.f, ki = 1.f, pi_ = 0.f, qi = 0.f;
-            if (i < M.nk) {
-                const float4 a4 = M.r32a[i];
-                const float4 b4 = M.r32b[i];
-                xi = a4.x; yi = a4.y; zi = a4.z; oi = b4.x; ki = b4.y; pi_ = b4.z; qi = b4.w;
+            for (int k = 0; k < NK; ++k) {
+                f16_scale(mx[k], sc[k], isc[k]);
+                if (part == 0) iscs[(slot * NK + k) * 128 + quad * 32 + lane] = isc[k];
             }
-            rc = RowF{xi, yi, zi, oi, ki, -pi_, -qi};
-            inv_cy = M.params[0];
-            until_flush = args.flush;
-        }
-        // this warp's 8 j: pair-packed records 4 part .. 4 part + 3
-        const float4* rec = reinterpret_cast<const float4*>(smem + L.rec_off + slot * 1024);
-        float2 t[4][2 * NK];
+            // the operand buffer is free once the MMAs of stage g - 2 are done
+            got = f16_wait(&mma_done[ab], ((g >> 1) & 1u) ^ 1u, args.err, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) break;
+            tc::fence_after();
+            // scaled FP16 hi / lo operand tiles of kind k: [hi Ta | lo Ta | hi Tb | lo Tb], 16
+            // columns each, this warp's NH of them
+            const uint32_t a = tmem + lane_off + f16_acol<NK, PPAD>(ab) + NH * part;
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const float4* v = rec + 4 * (4 * part + h);
-            f16_tiles2<NK>(kind0, rc, v[0], v[1], v[2], v[3], t[h]);
+            for (int k = 0; k < NK; ++k) {
 #pragma unroll
-            for (int k = 0; k < NK; ++k)  // the tiles that multiply y carry 1/c_y
-                t[h][2 * k + 1] = __fmul2_rn(t[h][2 * k + 1], make_float2(inv_cy, inv_cy));
+                for (int b = 0; b < 2; ++b) {
+#pragma unroll
+                    for (int h0 = 0; h0 < NH; h0 += 8) {
+                        uint32_t hw[8], lw[8];
+#pragma unroll
+                        for (int h = 0; h < 8; ++h)
+                            f16_split2(h0 + h < NS ? park[((h0 + h) * 2 + b) * 32] : t[h0 + h < NS ? 0 : h0 + h - NS][2 * k + b],
+                                       sc[k], hw[h], lw[h]);
+                        tc::st_x8(a + 64u * k + 32u * b + h0, hw);
+                        tc::st_x8(a + 64u * k + 32u * b + 16u + h0, lw);
+                    }
+                }
+            }
+            tc::wait_st();
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&a_full[ab]);  // this warp's operands and factors are in place
         }
-        // the row's largest |T| over the stage: this thread's 8 j, then the quad's 4 parts
-        const int xs = static_cast<int>(gs & 1u);
-        float* xrow = xm + (static_cast<size_t>((xs * 4 + quad) * NK) * 32 + lane) * 4;
+        tc::wait_st();  // nothing of ours is in flight to TMEM on any exit path
+    } else if (warp < kF16GenWarps + kF16DrainWarps) {
+        // ---------------------------------------------------------------- accumulator drain
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(f16_drain_regs<PPAD>()));
+        constexpr int CQ = PPAD / 2;  // accumulator columns per thread and kind
+        const int c_first = ((warp - kF16GenWarps) >> 2) * CQ;
+        float acc[NK][CQ];
 #pragma unroll
         for (int k = 0; k < NK; ++k)
-            xrow[k * 32 * 4 + part] = fmaxf(fmaxf(f16_absmax4(t[0][2 * k], t[1][2 * k]),
-                                                  f16_absmax4(t[2][2 * k], t[3][2 * k])),
-                                            fmaxf(f16_absmax4(t[0][2 * k + 1], t[1][2 * k + 1]),
-                                                  f16_absmax4(t[2][2 * k + 1], t[3][2 * k + 1])));
-        __syncwarp();  // the warp's 32 stores are ordered before lane 0's release
-        if (lane == 0) mbar_arrive(&xbar[xs * 4 + quad]);
-        got = f16_wait(&xbar[xs * 4 + quad], (gs >> 1) & 1u, args.err, abort_flag);
-        if (!__all_sync(0xffffffffu, got)) break;
-        float sc[NK], isc[NK];
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const float4 q = *reinterpret_cast<const float4*>(xrow + k * 32 * 4);
-            f16_scale(fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)), sc[k], isc[k]);
-        }
-        // scaled FP16 hi / lo operand tiles of kind k: [hi Ta | lo Ta | hi Tb | lo Tb], 16
-        // columns each; this warp's 8 j are columns 4 part .. 4 part + 3
-        const uint32_t a = tmem + lane_off + f16_acol<NK, PPAD>(ab) + 4 * part;
+            for (int c = 0; c < CQ; ++c) acc[k][c] = 0.0f;
+        int until_flush = args.flush;
+        for (uint32_t g = 0;; ++g) {
+            const int slot = g & 3, ab = g & 1;
+            bool got = f16_wait(&b_full[slot], (g >> 2) & 1u, args.err, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) break;
+            const F16Meta m = meta[slot];
+            if (m.flags & F16_END) break;
+            got = f16_wait(&mma_done[ab], (g >> 1) & 1u, args.err, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) break;
+            tc::fence_after();
+            float isc[NK];
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
+            for (int k = 0; k < NK; ++k) isc[k] = iscs[(slot * NK + k) * 128 + quad * 32 + lane];
+            __syncwarp();  // metadata and factors are read by every lane
+            if (lane == 0) mbar_arrive(&b_empty[slot]);
+            // into the FP32 registers, each value times the inverse row factor of the stage
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                uint32_t hw[4], lw[4];
+            for (int k = 0; k < NK; ++k) {
+                const uint32_t col = tmem + lane_off + f16_dcol<NK, PPAD>(k, ab) + c_first;
 #pragma unroll
-                for (int h = 0; h < 4; ++h) f16_split2(t[h][2 * k + b], sc[k], hw[h], lw[h]);
-                tc::st_x4(a + 64u * k + 32u * b, hw);
-                tc::st_x4(a + 64u * k + 32u * b + 16u, lw);
+                for (int c0 = 0; c0 < CQ; c0 += 8) {
+                    uint32_t r[8];
+                    tc::ld_x8(col + c0, r);
+                    tc::wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 8; c += 2) {
+                        const float2 v = __ffma2_rn(make_float2(__uint_as_float(r[c]), __uint_as_float(r[c + 1])),
+                                                    make_float2(isc[k], isc[k]),
+                                                    make_float2(acc[k][c0 + c], acc[k][c0 + c + 1]));
+                        acc[k][c0 + c] = v.x;
+                        acc[k][c0 + c + 1] = v.y;
+                    }
+                }
+            }
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_free[ab]);
+            if (m.flags & F16_FIRST) until_flush = args.flush;
+            if (--until_flush == 0 || (m.flags & F16_LAST)) {
+                // add the registers into the molecule's FP64 partial output (times 1/s_t; the
+                // gamma accumulator holds -(T3 u + T4 y)) and clear them
+                until_flush = args.flush;
+                const F16Mol& M = args.mols ? args.mols[m.mol] : args.single;
+                const int64_t i = static_cast<int64_t>(m.row_tile) * 128 + quad * 32 + lane;
+#pragma unroll
+                for (int k = 0; k < NK; ++k) {
+                    const int kind = NK == 2 ? k : m.kind;
+#pragma unroll
+                    for (int c = 0; c < CQ; ++c) {
+                        const int tr = c_first + c;
+                        if (i < M.nk && tr < M.Pn) {
+                            const int64_t tg = static_cast<int64_t>(M.t0) + tr;
+                            double* o = M.acc + ((static_cast<int64_t>(kind) * M.acc_P + tg) * M.nk_pad + i);
+                            const double v = static_cast<double>(acc[k][c]) * M.col_isc[tg];
+                            // streaming loads and stores: the partial output must not evict the
+                            // chunk's trial tiles from L2
+                            __stcs(o, __ldcs(o) + ((kind == 0) ? v : -v));
+                        }
+                        acc[k][c] = 0.0f;
+                    }
+                }
             }
         }
-        tc::wait_st();
-        tc::fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&a_full[ab]);  // this warp's operands are in place
-        // ---- MMA issue (one thread): this stage, once every warp's operands are in place
-        if (is_mma) {
-            bool go = f16_wait(&a_full[ab], aph, args.err, abort_flag);
-            if (go) {
+        tc::wait_ld();
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kF16RoleRegs));
+        if (warp == kF16ProducerWarp && lane == 0) {
+            // ------------------------------------------------------------ producer (one thread)
+            // keeps the ring full; every stage's copies complete on its b_full barrier together
+            // with this thread's arrival, which releases the metadata.
+            F16Cursor k;
+            f16_cursor_init<NK>(k, args);
+            if (!args.mols) {
+                tc::prefetch_tmap(&tm_bh);
+                tc::prefetch_tmap(&tm_bl);
+            }
+            int in_use = -1, unit = 0, ends = 0;
+            uint32_t g = 0;
+            for (; ends < 2; ++g) {
+                const int slot = g & 3;
+                if (!f16_wait(&b_empty[slot], ((g >> 2) & 1u) ^ 1u, args.err, abort_flag)) break;
+                if (k.done) {  // the end of the walk: a marker for each of the generating warpgroups
+                    meta[slot] = F16Meta{0, 0, 0, F16_END};
+                    mbar_arrive(&b_full[slot]);
+                    ++ends;
+                    continue;
+                }
+                const F16Mol& M = args.mols ? args.mols[k.mol] : args.single;
+                const CUtensorMap* mh = &tm_bh;
+                const CUtensorMap* ml = &tm_bl;
+                if (args.mols) {
+                    mh = M.maps;
+                    ml = M.maps + 1;
+                    if (k.mol != in_use) {  // a new molecule's tensor maps
+                        in_use = k.mol;
+                        tmap_acquire(mh);
+                        tmap_acquire(ml);
+                        tc::prefetch_tmap(mh);
+                        tc::prefetch_tmap(ml);
+                    }
+                }
+                const int s = k.s;
+                meta[slot] = F16Meta{k.mol, k.row_tile, k.kind,
+                                     (s == k.s0 ? F16_FIRST : 0) | (s == k.s1 - 1 ? F16_LAST : 0) | (unit << 3)};
+                if (s == k.s1 - 1) unit = (unit + 1) & 0xFFFFFFF;
+                uint8_t* base = smem + slot * L.slot_bytes;
+                uint8_t* rec = smem + L.rec_off + slot * 1024;
+                mbar_expect_tx(&b_full[slot], L.slot_bytes + 1024u);
+                bulk_g2s(rec, M.r32p + 2 * kF16Kj * static_cast<int64_t>(s), 1024u, &b_full[slot]);
+                // the chunk's trial tiles are re-read by every unit: keep them in L2 before other lines
+                const uint64_t pol = tc::l2_evict_last();
+                tc::tma_load_2d_hint(base, mh, 64 * s, M.t0, &b_full[slot], pol);
+                tc::tma_load_2d_hint(base + L.tile_bytes, ml, 64 * s, M.t0, &b_full[slot], pol);
+                f16_cursor_next<NK>(k, args);
+            }
+            // Copies in flight must land before the CTA exits: the last stages whose slots no
+            // end marker took (a marker is written after its slot's stage was consumed).
+            const uint32_t issued = g - ends, back = kF16Ring - ends;
+            for (uint32_t q = issued > back ? issued - back : 0; q < issued; ++q)
+                mbar_wait(&b_full[q & 3], (q >> 2) & 1u, args.err);
+        } else if (warp == kF16MmaWarp && lane == 0) {
+            // ------------------------------------------------------------ MMA issue (one thread)
+            // The tensor pipe's queue is short: the thread that issues a stage's MMAs is held for
+            // most of their run (960 of 1,250 cycles at Ppad = 192), so it does nothing else.
+            const uint32_t idesc = tc::idesc_f16(128, PPAD);
+            uint32_t g = 0;
+            for (;; ++g) {
+                const int slot = g & 3, ab = g & 1;
+                if (!f16_wait(&b_full[slot], (g >> 2) & 1u, args.err, abort_flag)) break;
+                if (meta[slot].flags & F16_END) break;
+                if (!f16_wait(&acc_free[ab], ((g >> 1) & 1u) ^ 1u, args.err, abort_flag)) break;
+                if (!f16_wait(&a_full[ab], (g >> 1) & 1u, args.err, abort_flag)) break;
                 tc::fence_after();
                 const uint32_t base = smem_u32(smem + slot * L.slot_bytes);
                 const uint64_t bh = tc::sdesc_kmajor_sw128(base);
@@ -571,7 +618,7 @@ k_hess_f16(const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CU
                 // K-step moves the descriptor's address field by 32 B (2 units)
 #pragma unroll
                 for (int k = 0; k < NK; ++k) {
-                    const uint32_t d = tmem + f16_dcol<NK, PPAD>(NK == 2 ? k : kind0, ab);
+                    const uint32_t d = tmem + f16_dcol<NK, PPAD>(k, ab);
                     const uint32_t aa = tmem + f16_acol<NK, PPAD>(ab) + 64u * k;
                     // operand tiles: Ta hi | Ta lo | Tb hi | Tb lo, 16 columns each (8 per
                     // 16-j half).  The small products first (the accumulator truncates its
@@ -591,56 +638,13 @@ k_hess_f16(const __grid_constant__ CUtensorMap tm_bh, const __grid_constant__ CU
                         tc::mma_f16_ts(d, aa + 32 + 8 * hh, bh + ky, idesc, 1u);  // Tb_hi y_hi
                     }
                 }
-                tc::commit(&mma_done[ab]);  // the ring slot is released after the drains
-                mma_any = true;
+                tc::commit(&mma_done[ab]);  // the ring slot is released by the drain warps
+            }
+            if (g > 0) {  // every MMA finished before TMEM is released
+                tc::commit(fin);
+                mbar_wait(fin, 0, args.err);
             }
         }
-        if (!__all_sync(0xffffffffu, !*abort_flag)) break;
-        // ---- drain the previous stage of this unit while this stage's MMAs run; then one
-        // more copy (one per drained stage: the slot it fills was drained a stage earlier)
-        if (!(m.flags & F16_FIRST)) {
-            if (!drain(dbuf, dph, kind0, isc_prev)) break;
-            if (lane == 0) mbar_arrive(&b_empty[pslot]);
-            if (--until_flush == 0) {
-                flush(mol, kind0, i);
-                until_flush = args.flush;
-            }
-            if (is_producer && !produce()) *abort_flag = 1;
-            if (!__all_sync(0xffffffffu, !*abort_flag)) break;
-        }
-#pragma unroll
-        for (int k = 0; k < NK; ++k) isc_prev[k] = isc[k];
-        dbuf = ab;
-        dph = aph;
-        pslot = slot;
-        if (++slot == kF16Ring) {
-            slot = 0;
-            ph ^= 1u;
-        }
-        ab ^= 1;
-        if (ab == 0) aph ^= 1u;
-        ++gs;
-        if (m.flags & F16_LAST) {  // the unit's last stage: drain it and write the rows out
-            if (!drain(dbuf, dph, kind0, isc_prev)) break;
-            if (lane == 0) mbar_arrive(&b_empty[pslot]);
-            if (is_producer && !produce()) *abort_flag = 1;
-            flush(mol, kind0, i);
-            if (!__all_sync(0xffffffffu, !*abort_flag)) break;
-        }
-    }
-    tc::wait_st();  // nothing of ours is in flight to TMEM on any exit path
-    tc::wait_ld();
-    if (is_producer) {  // copies in flight must land before the CTA exits
-        // (after the end marker, its slot's previous stage was drained before it was written,
-        // and that slot's parity has moved on: wait for the other ring slots only)
-        const int64_t issued = pr->issued;
-        const int64_t back = pr->end ? kF16Ring - 1 : kF16Ring;
-        for (int64_t k = (issued > back ? issued - back : 0); k < issued; ++k)
-            mbar_wait(&b_full[k % kF16Ring], static_cast<uint32_t>((k / kF16Ring) & 1), args.err);
-    }
-    if (is_mma && mma_any) {  // every MMA finished before TMEM is released
-        tc::commit(fin);
-        mbar_wait(fin, 0, args.err);
     }
     tc::fence_before();
     __syncthreads();
@@ -904,27 +908,27 @@ static bool f16_make_map(CUtensorMap* m, const void* base, int64_t nk_pad, int64
     return r == CUDA_SUCCESS;
 }
 
-template <int PQ, int NK>
+template <int PPAD, int NK>
 static cudaError_t launch_f16_t(const CUtensorMap* maps, const F16Args& a, int n_sm, cudaStream_t st) {
-    const F16Layout L = f16_layout(4 * PQ, NK);
-    cudaError_t e = cudaFuncSetAttribute(k_hess_f16<PQ, NK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const F16Layout L = f16_layout(PPAD, NK);
+    cudaError_t e = cudaFuncSetAttribute(k_hess_f16<PPAD, NK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L.total));
     if (e != cudaSuccess) return e;
     const int grid = static_cast<int>(a.n_units < n_sm ? a.n_units : n_sm);
     if (grid <= 0) return cudaSuccess;
-    k_hess_f16<PQ, NK><<<grid, kF16Threads, L.total, st>>>(maps[0], maps[1], a);
+    k_hess_f16<PPAD, NK><<<grid, kF16Threads, L.total, st>>>(maps[0], maps[1], a);
     return cudaGetLastError();
 }
 
 static cudaError_t launch_f16_dispatch(int ppad, const CUtensorMap* maps, const F16Args& a, int n_sm,
                                        cudaStream_t st) {
-    switch (ppad / 4) {
-        case 8: return launch_f16_t<8, 2>(maps, a, n_sm, st);
-        case 16: return launch_f16_t<16, 2>(maps, a, n_sm, st);
-        case 24: return launch_f16_t<24, 1>(maps, a, n_sm, st);
-        case 32: return launch_f16_t<32, 1>(maps, a, n_sm, st);
-        case 40: return launch_f16_t<40, 1>(maps, a, n_sm, st);
-        case 48: return launch_f16_t<48, 1>(maps, a, n_sm, st);
+    switch (ppad) {
+        case 32: return launch_f16_t<32, 2>(maps, a, n_sm, st);
+        case 64: return launch_f16_t<64, 2>(maps, a, n_sm, st);
+        case 96: return launch_f16_t<96, 1>(maps, a, n_sm, st);
+        case 128: return launch_f16_t<128, 1>(maps, a, n_sm, st);
+        case 160: return launch_f16_t<160, 1>(maps, a, n_sm, st);
+        case 192: return launch_f16_t<192, 1>(maps, a, n_sm, st);
         default: return cudaErrorInvalidValue;
     }
 }
