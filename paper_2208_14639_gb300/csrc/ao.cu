@@ -3,8 +3,9 @@
 //   M_mu_nu = sum_i w_i [s_i phi_mu phi_nu + 2 v_i . (phi_nu grad phi_mu + phi_mu grad phi_nu)]
 // with (s, v) = (f^rho, f^gamma grad rho) for F and (f^{rho,t}, f^{gamma,t} grad rho +
 // f^gamma grad rho^t) for G^t.  With Z_i,mu = w_i (s_i phi_i,mu / 2 + 2 v_i . grad phi_i,mu),
-// M = Phi^T Z + Z^T Phi: a plain FP64 GEMM over the kept points (this library's own split-K
-// kernel, gemm_f64.cu; the channels of a chunk side by side as the columns of one product),
+// M = Phi^T Z + Z^T Phi: a GEMM over the kept points (this library's own split-K kernels: exact
+// integer slices on the tensor cores, gemm_slices.cu, or FP64 FMA, gemm_f64.cu, where it is
+// short; the channels of a chunk side by side as the columns of one product),
 // then the symmetrisation.
 //
 // The nuclear derivative of the Fock matrix (Sec. II.B, F^a = F^a_G + F^a_gr + F^a_w, a = 3 A + c)
@@ -38,21 +39,22 @@ __global__ void k_ao_gather(PointsDev P, int32_t nbf, const double* __restrict__
     phik[e] = phi[P.orig[k] * nbf + mu];
 }
 
-// Z[k][c - c0][mu] (rows of nc x nbf) for the channels c0 .. c0 + nc - 1, nc = gridDim.y.
-// s: channel c's scalar at caller point i = s[c n + i]; the vector part is fg[c n + i]
-// grad rho_k (+ vg[i] gt[(c n + i) 3 + d] when gt is given).
-__global__ void k_ao_z(PointsDev P, int32_t nbf, const double* __restrict__ phi,
-                       const double* __restrict__ dphi, const double* __restrict__ s,
-                       const double* __restrict__ fg, const double* __restrict__ vg,
-                       const double* __restrict__ gt, int32_t c0, double* __restrict__ Z) {
+// Z is formed in two steps, so that no FP64 operation on a point and channel is repeated for every
+// basis function (GB300's FP64 pipe bounds this: 11 operations an element in one step, 5 in two):
+// coef[k][c - c0] = {a, b}, a = s / 2, b = 2 v for channel c, then Z[k][c - c0][mu] = w (a phi +
+// b . grad phi) (rows of nc x nbf).  (w stays outside: folded into the coefficients it adds a rounding
+// that all basis functions share, and the assembled matrices lose up to a factor four in accuracy.)
+// s: channel c's scalar at caller point i = s[c n + i]; v = fg[c n + i] grad rho_k (+ vg[i] gt[(c n +
+// i) 3 + d] when gt is given).  nc = gridDim.y.
+struct __align__(16) AoCoef { double a, x, y, z; };
+__global__ void k_ao_coef(PointsDev P, const double* __restrict__ s, const double* __restrict__ fg,
+                          const double* __restrict__ vg, const double* __restrict__ gt, int32_t c0,
+                          AoCoef* __restrict__ coef) {
     const int c = c0 + static_cast<int>(blockIdx.y);
-    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (e >= P.nk * nbf) return;
-    const int64_t k = e / nbf;
-    const int mu = static_cast<int>(e % nbf);
+    const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (k >= P.nk) return;
     const int64_t i = P.orig[k];
     const int64_t ci = static_cast<int64_t>(c) * P.n + i;
-    const double w = P.w[k];
     double vx = fg[ci] * P.gx[k], vy = fg[ci] * P.gy[k], vz = fg[ci] * P.gz[k];
     if (gt) {
         const double f = vg[i];
@@ -60,10 +62,26 @@ __global__ void k_ao_z(PointsDev P, int32_t nbf, const double* __restrict__ phi,
         vy += f * gt[3 * ci + 1];
         vz += f * gt[3 * ci + 2];
     }
-    const int64_t a = i * nbf + mu;
-    const double* d = dphi + 3 * a;
-    Z[(k * gridDim.y + blockIdx.y) * nbf + mu] =
-        w * (0.5 * s[ci] * phi[a] + 2.0 * (vx * d[0] + vy * d[1] + vz * d[2]));
+    coef[k * gridDim.y + blockIdx.y] = AoCoef{0.5 * s[ci], 2.0 * vx, 2.0 * vy, 2.0 * vz};
+}
+
+__global__ void __launch_bounds__(256)
+k_ao_z(PointsDev P, int32_t nbf, int32_t nc, bool weight, const double* __restrict__ phi,
+       const double* __restrict__ dphi, const AoCoef* __restrict__ coef, double* __restrict__ Z) {
+    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= P.nk * nbf) return;
+    const int64_t k = e / nbf;
+    const int mu = static_cast<int>(e % nbf);
+    const int64_t q = P.orig[k] * nbf + mu;
+    const double f = phi[q], dx = dphi[3 * q], dy = dphi[3 * q + 1], dz = dphi[3 * q + 2];
+    const double w = weight ? P.w[k] : 1.0;
+    const AoCoef* cf = coef + k * nc;
+    double* z = Z + k * nc * nbf + mu;
+#pragma unroll 4
+    for (int c = 0; c < nc; ++c) {
+        const AoCoef t = cf[c];
+        z[static_cast<int64_t>(c) * nbf] = w * fma(t.a, f, fma(t.z, dz, fma(t.y, dy, t.x * dx)));
+    }
 }
 
 // out[c] = M_c + M_c^T (M_c column-major nbf x nbf)
@@ -77,15 +95,12 @@ __global__ void k_ao_sym(int32_t nbf, const double* __restrict__ M, double* __re
     out[c * nn + e] = m[mu + static_cast<int64_t>(nu) * nbf] + m[nu + static_cast<int64_t>(mu) * nbf];
 }
 
-// Part (1) of the nuclear derivative: Z[k][a - a0][mu] = s^a phi / 2 + 2 v^a . grad phi for the
-// directions a0 .. a0 + gridDim.y - 1 (direction arrays: [a n + i], EUW_gr [(q n + i) P + a]).
-__global__ void k_fa_z(PointsDev P, FockDerivIn in, int32_t a0, double* __restrict__ Z) {
-    const int nbf = in.nbf;
+// Part (1) of the nuclear derivative: coef[k][a - a0] = {s^a / 2, 2 v^a} for the directions a0 ..
+// a0 + gridDim.y - 1 (direction arrays: [a n + i], EUW_gr [(q n + i) P + a]).
+__global__ void k_fa_coef(PointsDev P, FockDerivIn in, int32_t a0, AoCoef* __restrict__ coef) {
     const int a = a0 + static_cast<int>(blockIdx.y);
-    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (e >= P.nk * nbf) return;
-    const int64_t k = e / nbf;
-    const int mu = static_cast<int>(e % nbf);
+    const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (k >= P.nk) return;
     const int64_t i = P.orig[k];
     const int64_t ia = static_cast<int64_t>(a) * P.n + i;
     const int64_t np = static_cast<int64_t>(3) * P.n_atom;
@@ -99,13 +114,9 @@ __global__ void k_fa_z(PointsDev P, FockDerivIn in, int32_t a0, double* __restri
                      wa * fr;
     const double tg = w * (in.f_gamma_a[ia] + rho * P.om_g[k] * ww) + wa * fg;
     const double* ga = in.grad_rho_a + 3 * ia;
-    const double vx = tg * P.gx[k] + w * fg * ga[0];
-    const double vy = tg * P.gy[k] + w * fg * ga[1];
-    const double vz = tg * P.gz[k] + w * fg * ga[2];
-    const int64_t q = i * nbf + mu;
-    const double* d = in.dphi + 3 * q;
-    Z[(k * gridDim.y + blockIdx.y) * nbf + mu] =
-        0.5 * s * in.phi[q] + 2.0 * (vx * d[0] + vy * d[1] + vz * d[2]);
+    coef[k * gridDim.y + blockIdx.y] = AoCoef{0.5 * s, 2.0 * (tg * P.gx[k] + w * fg * ga[0]),
+                                              2.0 * (tg * P.gy[k] + w * fg * ga[1]),
+                                              2.0 * (tg * P.gz[k] + w * fg * ga[2])};
 }
 
 // Right factor of K^c (column-major nbf x 2 nk): column 2k = alpha phi + b . grad phi, column
@@ -177,32 +188,43 @@ int64_t ao_channels_per_chunk(int64_t nk, int32_t nbf, int32_t n_ch, size_t max_
 
 namespace {
 
-// Split count of one product, limited by the split-K scratch (work_elems doubles).
-int ao_splits(int M, int N, int64_t K, int n_sm, size_t work_elems) {
-    int s = gemm_abt_splits(M, N, K, n_sm);
+// One product C = A B^T (A M x K, B N x K, k slowest): on the tensor cores unless it is short.
+cudaError_t ao_product(const AoGemm& g, int M, int N, int64_t K, const double* A, const double* B,
+                       double* C, cudaStream_t st) {
+    if (gemm_slices_applies(K))
+        return launch_gemm_slices(M, N, K, A, M, B, N, C, M, g.work,
+                                  gemm_slices_splits(M, N, K, g.n_sm, g.work_elems), g.expo, g.err, st);
+    int s = gemm_abt_splits(M, N, K, g.n_sm);  // limited by the split-K scratch (work_elems doubles)
     const size_t per = static_cast<size_t>(M) * static_cast<size_t>(N);
-    const int cap = static_cast<int>(work_elems / (per > 0 ? per : 1));
-    return s < cap ? s : (cap > 0 ? cap : 1);
+    const int cap = static_cast<int>(g.work_elems / (per > 0 ? per : 1));
+    s = s < cap ? s : (cap > 0 ? cap : 1);
+    return launch_gemm_abt(M, N, K, A, M, B, N, C, M, g.work, s, st);
 }
 
-// The channel chunks of M = Phi^T Z + Z^T Phi: make_z(c0, nc) launches the kernel that writes Z
-// for channels c0 .. c0 + nc - 1; phik holds the gathered basis values.
-template <class MakeZ>
+// The channel chunks of M = Phi^T Z + Z^T Phi: make_coef(c0, nc, coef) launches the kernel that writes
+// the coefficients of channels c0 .. c0 + nc - 1; phik holds the gathered basis values; Z has
+// room for chunk nk (nbf + 4) + 1 doubles.  weight: Z carries the quadrature weight (else the
+// coefficients do).
+template <class MakeCoef>
 cudaError_t assemble_chunks(const PointsDev& p, const AoGemm& g, int32_t nbf, int32_t n_ch,
-                            int64_t chunk, const double* phik, double* Z, double* M, double* out,
-                            cudaStream_t st, MakeZ make_z) {
+                            int64_t chunk, bool weight, const double* phi, const double* dphi,
+                            const double* phik, double* Z, double* M, double* out, cudaStream_t st, MakeCoef make_coef) {
     const int64_t nn = static_cast<int64_t>(nbf) * nbf;
+    // after Z, on a 16-byte boundary (nk nbf chunk may be odd)
+    AoCoef* coef = reinterpret_cast<AoCoef*>(Z + ((p.nk * nbf * chunk + 1) & ~int64_t(1)));
     for (int32_t c0 = 0; c0 < n_ch; c0 += static_cast<int32_t>(chunk)) {
         const int32_t nc = static_cast<int32_t>(n_ch - c0 < chunk ? n_ch - c0 : chunk);
-        make_z(c0, nc);
+        make_coef(c0, nc, coef);
         cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        k_ao_z<<<static_cast<unsigned>((p.nk * nbf + 255) / 256), 256, 0, st>>>(p, nbf, nc, weight, phi, dphi,
+                                                                                coef, Z);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         // one product for the chunk: M (column-major nbf x nc nbf) = A B^T with A = phik
         // viewed as nbf x nk and B = Z viewed as (nc nbf) x nk (k slowest in both); column
         // c nbf + nu of M is column nu of M_c
-        const int N = nc * nbf;
-        e = launch_gemm_abt(nbf, N, p.nk, phik, nbf, Z, N, M, nbf, g.work,
-                            ao_splits(nbf, N, p.nk, g.n_sm, g.work_elems), st);
+        e = ao_product(g, nbf, nc * nbf, p.nk, phik, Z, M, st);
         if (e != cudaSuccess) return e;
         k_ao_sym<<<dim3(static_cast<unsigned>((nn + 255) / 256), static_cast<unsigned>(nc)), 256, 0, st>>>(
             nbf, M, out + c0 * nn);
@@ -226,10 +248,10 @@ cudaError_t launch_ao_assemble(const PointsDev& p, const AoGemm& g, int32_t nbf,
     k_ao_gather<<<gx, 256, 0, st>>>(p, nbf, phi, phik);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return assemble_chunks(p, g, nbf, n_ch, chunk, phik, Z, M, out, st,
-                           [&](int32_t c0, int32_t nc) {
-                               k_ao_z<<<dim3(gx, static_cast<unsigned>(nc)), 256, 0, st>>>(
-                                   p, nbf, phi, dphi, s, fg, vg, gt, c0, Z);
+    return assemble_chunks(p, g, nbf, n_ch, chunk, true, phi, dphi, phik, Z, M, out, st,
+                           [&](int32_t c0, int32_t nc, AoCoef* coef) {
+                               k_ao_coef<<<dim3(static_cast<unsigned>((p.nk + 255) / 256), static_cast<unsigned>(nc)),
+                                           256, 0, st>>>(p, s, fg, vg, gt, c0, coef);
                            });
 }
 
@@ -247,9 +269,10 @@ cudaError_t launch_fock_derivative(const PointsDev& p, const AoGemm& g, const Fo
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // (1) the terms without derivatives of the basis functions (writes every out[a])
-    e = assemble_chunks(p, g, nbf, n_dir, chunk, phik, Z, M, out, st,
-                        [&](int32_t a0, int32_t nc) {
-                            k_fa_z<<<dim3(gx, static_cast<unsigned>(nc)), 256, 0, st>>>(p, in, a0, Z);
+    e = assemble_chunks(p, g, nbf, n_dir, chunk, false, in.phi, in.dphi, phik, Z, M, out, st,
+                        [&](int32_t a0, int32_t nc, AoCoef* coef) {
+                            k_fa_coef<<<dim3(static_cast<unsigned>((p.nk + 255) / 256), static_cast<unsigned>(nc)),
+                                        256, 0, st>>>(p, in, a0, coef);
                         });
     if (e != cudaSuccess) return e;
     // (2) the derivatives of the basis functions
@@ -264,14 +287,12 @@ cudaError_t launch_fock_derivative(const PointsDev& p, const AoGemm& g, const Fo
         k_fa_left<<<gx, 256, 0, st>>>(p, in, c, L);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = launch_gemm_abt(nbf, nbf, 2 * p.nk, L, nbf, R, nbf, Kall, nbf, g.work,
-                            ao_splits(nbf, nbf, 2 * p.nk, g.n_sm, g.work_elems), st);
+        e = ao_product(g, nbf, nbf, 2 * p.nk, L, R, Kall, st);
         if (e != cudaSuccess) return e;
         for (int32_t A = 0; A < p.n_atom; ++A) {
             const int64_t s0 = seg[A], na = seg[A + 1] - seg[A];
             if (na > 0) {
-                e = launch_gemm_abt(nbf, nbf, 2 * na, L + 2 * s0 * nbf, nbf, R + 2 * s0 * nbf, nbf,
-                                    KA, nbf, g.work, ao_splits(nbf, nbf, 2 * na, g.n_sm, g.work_elems), st);
+                e = ao_product(g, nbf, nbf, 2 * na, L + 2 * s0 * nbf, R + 2 * s0 * nbf, KA, st);
                 if (e != cudaSuccess) return e;
             }
             k_fa_basis<<<gn, 256, 0, st>>>(nbf, A, in.bf_atom, Kall, na > 0 ? KA : nullptr,

@@ -387,14 +387,27 @@ cudaError_t launch_gemm_abt(int M, int N, int64_t K, const double* A, int64_t ld
                             int64_t ldb, double* C, int64_t ldc, double* work, int n_split,
                             cudaStream_t st);
 
+// The same product on the tensor cores, as exact integer slice products (gemm_slices.cu); work as
+// above, expo: gemm_slices_expo_ints(M + N, K), err: the device error word.
+// gemm_slices_applies: where it is faster.
+size_t gemm_slices_expo_ints(int64_t rows, int64_t K);
+bool gemm_slices_applies(int64_t K);
+int gemm_slices_splits(int M, int N, int64_t K, int n_sm, size_t work_elems);
+cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t lda, const double* B,
+                               int64_t ldb, double* C, int64_t ldc, double* work, int n_split,
+                               int32_t* expo, int* err, cudaStream_t st);
+
 // AO-side assembly (Sec. II.A Fock matrix, Sec. II.B contracted orbital Hessian): out[c] =
 // M_c + M_c^T, M_c = Phi^T Z_c over the kept points, channels in chunks of `chunk`
-// (ao_channels_per_chunk).  Scratch: phik (nk x nbf), Z (chunk x nk x nbf), M (chunk x nbf x
-// nbf) and the product's split-K partials (AoGemm: ao_gemm_work_elems doubles).
+// (ao_channels_per_chunk).  Scratch: phik (nk x nbf), Z and its coefficients (chunk x nk x (nbf +
+// 4), + 1), M (chunk x nbf x nbf) and the product's split-K partials (AoGemm: ao_gemm_work_elems
+// doubles, and the exponents of a product of (chunk + 1) nbf rows over 2 nk points).
 struct AoGemm {
     double* work;
     size_t work_elems;
+    int32_t* expo;
     int n_sm;
+    int* err;
 };
 size_t ao_gemm_work_elems(int32_t nbf, int64_t chunk, int n_sm);
 int64_t ao_channels_per_chunk(int64_t nk, int32_t nbf, int32_t n_ch, size_t max_bytes);
