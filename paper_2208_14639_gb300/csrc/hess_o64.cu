@@ -24,8 +24,12 @@
 // factors' inverses (powers of two) and adds it into a double-FP32 register sum per output;
 // the flush adds that sum in FP64 to the partial output.
 //
-// Work unit: 128 rows x one output kind x the trials of the launch (MMA N = Ppad = 32; TMEM
-// holds 7 x 32 accumulator and 7 x 16 operand columns).  The j range is walked in L2-sized
+// Work unit: 128 rows x one output kind x the trials of the launch (MMA N = Ppad, 32, 48 or 64:
+// TMEM holds 7 Ppad accumulator and 7 x 16 operand columns, at 64 the last three slices' operands
+// in shared memory).  The tiles, some 420 FP32 operations per pair and kind, bound the kernel (FMA
+// pipe), so a launch takes as many trials as the accumulators allow (39,542 points, P = 36: 145 ms
+// in two launches of 18 with whole units per CTA, 80 in one, 61 with equal shares of the stages;
+// 29,778 points, P = 54: 88, 56, 44).  The j range is walked in L2-sized
 // chunks as in the split-FP16 kernel (each CTA its fixed units in every chunk).  16 warps (4
 // per TMEM lane quadrant, 4 j each): generate the two tiles of the row, exchange the stage's
 // row maxima, wait for the previous stage's MMAs and drain them, slice and store the operands
@@ -48,8 +52,10 @@ constexpr int kO64Threads = kO64Warps * 32;
 constexpr int kO64Ring = 4;         // stages of copies in flight
 constexpr int kO64Slices = 7;
 constexpr int kO64Levels = 7;       // p + q = 0 .. 6
-constexpr int kO64Ppad = 32;        // trials per launch (MMA N)
-constexpr int kO64PQ = kO64Ppad / 4;
+constexpr int kO64MaxPpad = 64;      // trials per launch (MMA N): 32, 48 or 64
+// Tile slices that do not fit the TMEM beside the accumulators (7 Ppad columns): the last ones, which
+// enter the fewest products (6 of 28), are read from shared memory.
+constexpr int o64_smem_slices(int ppad) { return ppad > 48 ? 3 : 0; }
 constexpr uint32_t kO64TmemCols = 512;
 constexpr size_t kO64ChunkBytes = 48u << 20;
 constexpr uint32_t kO64RecBytes = 64;  // one column record (FP32 pairs)
@@ -59,17 +65,19 @@ struct O64Layout {
     uint32_t slot_bytes;  // the seven slice tiles of one stage
     uint32_t civ_off;     // the stage's column-factor inverses [Ppad] floats, per ring slot
     uint32_t rec_off;     // the stage's 16 column records, per ring slot
+    uint32_t a_off;       // the tile slices kept in shared memory, 128 64-byte rows each
     uint32_t xm_off;      // row-maximum exchange [2][4 quads][32 lanes][4 parts] floats
     uint32_t prod_off;    // the producer thread's state
     uint32_t bar_off;
     uint32_t total;
 };
-__host__ __device__ constexpr O64Layout o64_layout() {
+__host__ __device__ constexpr O64Layout o64_layout(int ppad) {
     O64Layout L{};
-    L.tile_bytes = kO64Ppad * 64u;
+    L.tile_bytes = static_cast<uint32_t>(ppad) * 64u;
     L.slot_bytes = kO64Slices * L.tile_bytes;
-    L.civ_off = kO64Ring * L.slot_bytes;
-    L.rec_off = L.civ_off + kO64Ring * kO64Ppad * 4u;
+    L.a_off = kO64Ring * L.slot_bytes;
+    L.civ_off = L.a_off + o64_smem_slices(ppad) * 128u * 64u;
+    L.rec_off = L.civ_off + kO64Ring * static_cast<uint32_t>(ppad) * 4u;
     L.xm_off = L.rec_off + kO64Ring * kO64Kj * kO64RecBytes;
     L.prod_off = L.xm_off + 2u * 4u * 32u * 4u * 4u;
     L.bar_off = L.prod_off + 128u;
@@ -95,9 +103,11 @@ struct O64Args {
     int64_t nk, nk_pad, acc_P;
     int32_t Pn, t0;
     int64_t n_units;         // row tiles x 2 output kinds
-    int32_t n_stage, chunk;
+    int32_t n_stage, chunk;  // chunk = 0: the stages of all units in one line, an equal share per CTA
     int32_t flush;
+    double* side;            // chunk = 0: [CTA][Pn][128] partial output of a share's first, begun unit
     int* err;
+    __host__ __device__ int64_t first(int64_t cta, int64_t grid) const { return cta * (n_units * n_stage) / grid; }
 };
 
 struct O64Cursor {
@@ -111,12 +121,20 @@ struct O64Prod {
     int32_t slot;
     uint32_t ph, end;
 };
-enum : int32_t { O64_FIRST = 1, O64_LAST = 2, O64_END = 4 };
+enum : int32_t { O64_FIRST = 1, O64_LAST = 2, O64_END = 4, O64_SIDE = 8 };
 struct O64Meta {
     int32_t row_tile, kind, flags, pad;
 };
 
 __device__ __forceinline__ void o64_cursor_init(O64Cursor& k, const O64Args& a) {
+    if (a.chunk == 0) {
+        const int64_t b = a.first(blockIdx.x, gridDim.x), e = a.first(blockIdx.x + 1, gridDim.x);
+        k.u = b / a.n_stage;
+        k.s = k.s0 = static_cast<int>(b - k.u * a.n_stage);
+        k.s1 = static_cast<int>(min(static_cast<int64_t>(a.n_stage), k.s0 + (e - b)));
+        k.done = b >= e;
+        return;
+    }
     k.c = 0;
     k.u = blockIdx.x;
     k.s0 = 0;
@@ -126,6 +144,13 @@ __device__ __forceinline__ void o64_cursor_init(O64Cursor& k, const O64Args& a) 
 }
 __device__ __forceinline__ void o64_cursor_next(O64Cursor& k, const O64Args& a) {
     if (++k.s < k.s1) return;
+    if (a.chunk == 0) {  // on to the next unit of the share
+        const int64_t left = a.first(blockIdx.x + 1, gridDim.x) - (++k.u) * a.n_stage;
+        k.s = k.s0 = 0;
+        k.s1 = static_cast<int>(min(static_cast<int64_t>(a.n_stage), left));
+        k.done = left <= 0;
+        return;
+    }
     k.u += gridDim.x;
     if (k.u >= a.n_units) {
         k.u = blockIdx.x;
@@ -337,24 +362,26 @@ __device__ __forceinline__ void o64_slices(float hi, float lo, float (&s)[kO64Sl
     s[6] = rintf(fmaf(w.l, 281474976710656.0f, (u5 - s[5]) * 256.0f));  // w.l 2^48
 }
 
-// TMEM columns: level l accumulator at 32 l (l = 0..6); operand slices at 224: slice p, tile
-// b (0: Ta, 1: Tb) at 224 + 16 p + 8 b, 8 columns (16 j, two FP16 each).
-__device__ __forceinline__ uint32_t o64_dcol(int l) { return static_cast<uint32_t>(kO64Ppad * l); }
-__device__ __forceinline__ uint32_t o64_acol(int p, int b) {
-    return static_cast<uint32_t>(kO64Levels * kO64Ppad + 16 * p + 8 * b);
+// TMEM columns: level l accumulator at Ppad l (l = 0..6); operand slices behind them: slice p, tile
+// b (0: Ta, 1: Tb) at 7 Ppad + 16 p + 8 b, 8 columns (16 j, two FP16 each).
+template <int PPAD> __device__ __forceinline__ uint32_t o64_dcol(int l) { return static_cast<uint32_t>(PPAD * l); }
+template <int PPAD> __device__ __forceinline__ uint32_t o64_acol(int p, int b) {
+    return static_cast<uint32_t>(kO64Levels * PPAD + 16 * p + 8 * b);
 }
-static_assert(kO64Levels * kO64Ppad + 16 * kO64Slices <= static_cast<int>(kO64TmemCols), "TMEM");
 
+template <int PPAD>
 __global__ void __launch_bounds__(kO64Threads, 1)
 k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
            const __grid_constant__ CUtensorMap tm2, const __grid_constant__ CUtensorMap tm3,
            const __grid_constant__ CUtensorMap tm4, const __grid_constant__ CUtensorMap tm5,
            const __grid_constant__ CUtensorMap tm6, O64Args args) {
-    constexpr int PQ = kO64PQ;
+    constexpr int PQ = PPAD / 4;
+    constexpr int kTm = kO64Slices - o64_smem_slices(PPAD);  // tile slices in TMEM
+    static_assert(kO64Levels * PPAD + 16 * kTm <= static_cast<int>(kO64TmemCols), "TMEM");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    constexpr O64Layout L = o64_layout();
+    constexpr O64Layout L = o64_layout(PPAD);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bar_off);
     uint64_t* b_full = bars;                    // [kO64Ring]
     uint64_t* b_empty = bars + kO64Ring;        // [kO64Ring]
@@ -406,12 +433,13 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
         }
         const int s = P.k.s;
         meta[P.slot] = O64Meta{static_cast<int32_t>(P.k.u >> 1), static_cast<int32_t>(P.k.u & 1),
-                               (s == P.k.s0 ? O64_FIRST : 0) | (s == P.k.s1 - 1 ? O64_LAST : 0), 0};
-        constexpr uint32_t rec_bytes = kO64Kj * kO64RecBytes, civ_bytes = kO64Ppad * 4u;
+                               (s == P.k.s0 ? O64_FIRST : 0) | (s == P.k.s1 - 1 ? O64_LAST : 0) |
+                                   (args.chunk == 0 && P.k.s0 > 0 ? O64_SIDE : 0), 0};
+        constexpr uint32_t rec_bytes = kO64Kj * kO64RecBytes, civ_bytes = PPAD * 4u;
         mbar_expect_tx(&b_full[P.slot], L.slot_bytes + rec_bytes + civ_bytes);
         bulk_g2s(smem + L.rec_off + P.slot * rec_bytes, args.rec + static_cast<int64_t>(kO64Kj / 2) * s,
                  rec_bytes, &b_full[P.slot]);  // the stage's kO64Kj / 2 pair records
-        bulk_g2s(smem + L.civ_off + P.slot * civ_bytes, args.civ + static_cast<int64_t>(kO64Ppad) * s,
+        bulk_g2s(smem + L.civ_off + P.slot * civ_bytes, args.civ + static_cast<int64_t>(PPAD) * s,
                  civ_bytes, &b_full[P.slot]);
         uint8_t* base = smem + P.slot * L.slot_bytes;
         for (int q = 0; q < kO64Slices; ++q)
@@ -437,7 +465,7 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
     }
 
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const uint32_t idesc = tc::idesc_f16(128, kO64Ppad);
+    const uint32_t idesc = tc::idesc_f16(128, PPAD);
     const float inv_cy = static_cast<float>(args.params[0]);  // a power of two
     float ahi[PQ], alo[PQ];  // double-FP32 sums of this thread's columns
 #pragma unroll
@@ -454,7 +482,7 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
             uint32_t r[kO64Levels][4];
 #pragma unroll
             for (int l = 0; l < kO64Levels; ++l)
-                tc::ld_x4(tmem + lane_off + o64_dcol(l) + part * PQ + c0, r[l]);
+                tc::ld_x4(tmem + lane_off + o64_dcol<PPAD>(l) + part * PQ + c0, r[l]);
             tc::wait_ld();
             const float4 cv = *reinterpret_cast<const float4*>(civ + part * PQ + c0);
             const float cf[4] = {cv.x, cv.y, cv.z, cv.w};
@@ -478,13 +506,15 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
         tc::fence_before();
         return true;
     };
-    auto flush = [&](int kind, int64_t i) {
+    auto flush = [&](int kind, bool side, int64_t i) {
+        double* base = side ? args.side + static_cast<int64_t>(blockIdx.x) * args.Pn * 128 + (i & 127)
+                            : args.acc + (static_cast<int64_t>(kind) * args.acc_P + args.t0) * args.nk_pad + i;
+        const int64_t ld = side ? 128 : args.nk_pad;
 #pragma unroll
         for (int c = 0; c < PQ; ++c) {
             const int t = part * PQ + c;
             if (i < args.nk && t < args.Pn) {
-                const int64_t tg = static_cast<int64_t>(args.t0) + t;
-                double* o = args.acc + ((static_cast<int64_t>(kind) * args.acc_P + tg) * args.nk_pad + i);
+                double* o = base + t * ld;
                 const double v = static_cast<double>(ahi[c]) + static_cast<double>(alo[c]);
                 __stcs(o, __ldcs(o) + ((kind == 0) ? v : -v));  // streaming: keep the tiles in L2
             }
@@ -560,11 +590,11 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
         // drain them before the operands are overwritten
         if (pending) {
             if (!drain(mph ^ 1u, riv_prev,
-                       reinterpret_cast<const float*>(smem + L.civ_off + pslot * kO64Ppad * 4)))
+                       reinterpret_cast<const float*>(smem + L.civ_off + pslot * PPAD * 4)))
                 break;
             if (lane == 0) mbar_arrive(&b_empty[pslot]);
             if (--until_flush == 0) {
-                flush(kind0, i);
+                flush(kind0, (m.flags & O64_SIDE) != 0, i);
                 until_flush = args.flush;
             }
             if (is_producer && !pr->end && !produce()) *abort_flag = 1;
@@ -585,11 +615,18 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
             for (int p = 0; p < kO64Slices; ++p) {
                 const __half2 x = __floats2half2_rn(s0[p], s1[p]);
                 const __half2 y = __floats2half2_rn(s2[p], s3[p]);
-                tc::st_x2(a + o64_acol(p, b), *reinterpret_cast<const uint32_t*>(&x),
-                          *reinterpret_cast<const uint32_t*>(&y));
+                const uint32_t xw = *reinterpret_cast<const uint32_t*>(&x), yw = *reinterpret_cast<const uint32_t*>(&y);
+                if (p < kTm) {
+                    tc::st_x2(a + o64_acol<PPAD>(p, b), xw, yw);
+                } else {  // halves 16 b + 4 part .. of the row, 64-byte swizzle
+                    const int r = quad * 32 + lane, chunk = (2 * b + (part >> 1)) ^ ((r >> 1) & 3);
+                    *reinterpret_cast<uint2*>(smem + L.a_off + (p - kTm) * 8192 + r * 64 + chunk * 16 + (part & 1) * 8) =
+                        make_uint2(xw, yw);
+                }
             }
         }
         tc::wait_st();
+        if (kTm < kO64Slices) tc::fence_proxy_async_smem();
         tc::fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(a_full);
@@ -601,12 +638,18 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
                 // trial rows: [u' (16 j) | c_y y' (16 j)], 32 B each (2 descriptor units)
 #pragma unroll
                 for (int l = 0; l < kO64Levels; ++l) {
-                    const uint32_t d = tmem + o64_dcol(l);
+                    const uint32_t d = tmem + o64_dcol<PPAD>(l);
 #pragma unroll
                     for (int p = 0; p <= l; ++p) {
                         const uint64_t bd = tc::sdesc_kmajor_sw64(base + (l - p) * L.tile_bytes);
-                        tc::mma_f16_ts(d, tmem + o64_acol(p, 0), bd, idesc, p == 0 ? 0u : 1u);
-                        tc::mma_f16_ts(d, tmem + o64_acol(p, 1), bd + 2u, idesc, 1u);
+                        if (p < kTm) {
+                            tc::mma_f16_ts(d, tmem + o64_acol<PPAD>(p, 0), bd, idesc, p == 0 ? 0u : 1u);
+                            tc::mma_f16_ts(d, tmem + o64_acol<PPAD>(p, 1), bd + 2u, idesc, 1u);
+                        } else {
+                            const uint64_t ad = tc::sdesc_kmajor_sw64(smem_u32(smem + L.a_off) + (p - kTm) * 8192u);
+                            tc::mma_f16_ss(d, ad, bd, idesc, 1u);
+                            tc::mma_f16_ss(d, ad + 2u, bd + 2u, idesc, 1u);
+                        }
                     }
                 }
                 tc::commit(mma_done);
@@ -625,12 +668,12 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
         ++gs;
         if (m.flags & O64_LAST) {  // the unit's last stage: drain it and write the rows out
             if (!drain(mph ^ 1u, riv_prev,
-                       reinterpret_cast<const float*>(smem + L.civ_off + pslot * kO64Ppad * 4)))
+                       reinterpret_cast<const float*>(smem + L.civ_off + pslot * PPAD * 4)))
                 break;
             if (lane == 0) mbar_arrive(&b_empty[pslot]);
             if (is_producer && !pr->end && !produce()) *abort_flag = 1;
             pending = false;
-            flush(kind0, i);
+            flush(kind0, (m.flags & O64_SIDE) != 0, i);
             if (!__all_sync(0xffffffffu, !*abort_flag)) break;
         }
     }
@@ -654,6 +697,26 @@ k_hess_o64(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUte
         tc::fence_after();
         tc::tmem_dealloc(tmem, kO64TmemCols);
     }
+}
+
+// Equal shares: adds the side outputs of the CTAs that began inside a unit to the unit's partial
+// output, in CTA order.  Thread = (unit, trial, row).
+__global__ void __launch_bounds__(128) k_o64_join(O64Args a, int32_t grid) {
+    const int64_t u = blockIdx.x;
+    const int t = blockIdx.y;
+    const int64_t i = (u >> 1) * 128 + threadIdx.x;
+    if (i >= a.nk) return;
+    const int64_t b = u * a.n_stage, all = a.n_units * a.n_stage;
+    double v = 0.0;
+    // shares with b < first(c) < b + n_stage (first(c) = floor(c all / grid))
+    for (int64_t c = (b * grid) / all; c < grid; ++c) {
+        const int64_t f = a.first(c, grid);
+        if (f <= b) continue;
+        if (f >= b + a.n_stage) break;
+        v += a.side[(c * a.Pn + t) * 128 + threadIdx.x];
+    }
+    double* o = a.acc + ((u & 1) * a.acc_P + a.t0 + t) * a.nk_pad + i;
+    *o += v;
 }
 
 // ---------------------------------------------------------------- records and trial slices
@@ -727,11 +790,11 @@ __global__ void k_o64_balance(const unsigned long long* __restrict__ colmax,
 
 // The seven FP16 slice arrays [rows][2 nk_pad] (per 16-j block: 16 u' then 16 c_y y', scaled by
 // the block's column factor; slices exact in FP64) and the factors' inverses
-// civ[group][n_stage][32] for trial groups [g pg, g pg + pg): one half-warp per (trial, 16-j
+// civ[group][n_stage][ppad] for trial groups [g pg, g pg + pg): one half-warp per (trial, 16-j
 // block).  Rows t >= P are zero.
 __global__ void __launch_bounds__(256)
 k_o64_split(const double* __restrict__ u, const double* __restrict__ y, int32_t P, int32_t pg,
-            int64_t nk_pad, const double* __restrict__ params, __half* __restrict__ out,
+            int32_t ppad, int64_t nk_pad, const double* __restrict__ params, __half* __restrict__ out,
             int64_t slice_stride, float* __restrict__ civ) {
     const int t = blockIdx.y;
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;  // < nk_pad
@@ -761,7 +824,7 @@ k_o64_split(const double* __restrict__ u, const double* __restrict__ y, int32_t 
     if (t < P && (j & 15) == 0) {
         const int g = t / pg, c = t - g * pg;
         const int64_t n_stage = nk_pad / kO64Kj;
-        civ[(static_cast<int64_t>(g) * n_stage + (j >> 4)) * kO64Ppad + c] = isc;
+        civ[(static_cast<int64_t>(g) * n_stage + (j >> 4)) * ppad + c] = isc;
     }
 }
 
@@ -782,13 +845,13 @@ static PFN_cuTensorMapEncodeTiled_v12000 o64_encode_fn() {
     return fn;
 }
 
-// [rows][2 nk_pad] halves; box 32 halves (one stage: 16 u', 16 c_y y') x 32 rows, 64-byte swizzle.
-static bool o64_make_map(CUtensorMap* m, const void* base, int64_t nk_pad, int64_t rows) {
+// [rows][2 nk_pad] halves; box 32 halves (one stage: 16 u', 16 c_y y') x ppad rows, 64-byte swizzle.
+static bool o64_make_map(CUtensorMap* m, const void* base, int64_t nk_pad, int64_t rows, int ppad) {
     auto fn = o64_encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {static_cast<cuuint64_t>(2 * nk_pad), static_cast<cuuint64_t>(rows)};
     cuuint64_t strides[1] = {static_cast<cuuint64_t>(2 * nk_pad) * sizeof(__half)};
-    cuuint32_t box[2] = {32u, static_cast<cuuint32_t>(kO64Ppad)};
+    cuuint32_t box[2] = {32u, static_cast<cuuint32_t>(ppad)};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides,
                     box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
@@ -796,10 +859,11 @@ static bool o64_make_map(CUtensorMap* m, const void* base, int64_t nk_pad, int64
     return r == CUDA_SUCCESS;
 }
 
-int hess_o64_max_group() { return kO64Ppad; }
+int hess_o64_max_group() { return kO64MaxPpad; }
+int hess_o64_ppad(int32_t Pn) { return Pn <= 32 ? 32 : (Pn <= 48 ? 48 : 64); }
 int hess_o64_slices() { return kO64Slices; }
 int64_t hess_o64_civ_floats(int32_t P, int32_t pg, int64_t nk_pad) {
-    return static_cast<int64_t>((P + pg - 1) / pg) * (nk_pad / kO64Kj) * kO64Ppad;
+    return static_cast<int64_t>((P + pg - 1) / pg) * (nk_pad / kO64Kj) * hess_o64_ppad(pg);
 }
 
 cudaError_t launch_o64_prep(const PointsDev& p, const double* u, const double* y, int32_t P,
@@ -807,35 +871,56 @@ cudaError_t launch_o64_prep(const PointsDev& p, const double* u, const double* y
                             double* params, void* slices, int64_t slice_stride, float* civ,
                             cudaStream_t st) {
     const int64_t nk_pad = p.nk_pad;
-    if (nk_pad % 256 != 0 || pg < 1 || pg > kO64Ppad) return cudaErrorInvalidValue;
-    const int ng = (P + pg - 1) / pg;
+    if (nk_pad % 256 != 0 || pg < 1 || pg > kO64MaxPpad) return cudaErrorInvalidValue;
+    const int ppad = hess_o64_ppad(pg), ng = (P + pg - 1) / pg;
     const int64_t nb = nk_pad / 256;
     k_o64_records<<<static_cast<unsigned>(nb), 256, 0, st>>>(p.r64a, p.r64b, nk_pad,
                                                               static_cast<O64Rec*>(rec));  // nk_pad / 2 pair records
     cudaError_t e = cudaMemsetAsync(colmax, 0, 2 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     // zero factors for the padding columns of every group
-    e = cudaMemsetAsync(civ, 0, sizeof(float) * static_cast<size_t>(ng) * (nk_pad / kO64Kj) * kO64Ppad, st);
+    e = cudaMemsetAsync(civ, 0, sizeof(float) * static_cast<size_t>(ng) * (nk_pad / kO64Kj) * ppad, st);
     if (e != cudaSuccess) return e;
     dim3 g1(static_cast<unsigned>(nb < 16 ? nb : 16), static_cast<unsigned>(P));
     k_o64_colmax<<<g1, 256, 0, st>>>(u, y, nk_pad, colmax);
     k_o64_balance<<<1, 1, 0, st>>>(colmax, params);
     dim3 g2(static_cast<unsigned>(nb), static_cast<unsigned>(rows));
-    k_o64_split<<<g2, 256, 0, st>>>(u, y, P, pg, nk_pad, params, static_cast<__half*>(slices),
+    k_o64_split<<<g2, 256, 0, st>>>(u, y, P, pg, ppad, nk_pad, params, static_cast<__half*>(slices),
                                     slice_stride, civ);
+    return cudaGetLastError();
+}
+
+template <int PPAD>
+static cudaError_t o64_launch(const CUtensorMap* maps, const O64Args& a, int n_sm, cudaStream_t st) {
+    constexpr O64Layout L = o64_layout(PPAD);
+    cudaError_t e = cudaFuncSetAttribute(k_hess_o64<PPAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(L.total));
+    if (e != cudaSuccess) return e;
+    const int64_t work = a.chunk == 0 ? a.n_units * a.n_stage / 8 : a.n_units;  // >= 8 stages a share
+    const int grid = static_cast<int>(work < n_sm ? work : n_sm);
+    if (a.chunk == 0) {
+        e = cudaMemsetAsync(a.side, 0, sizeof(double) * 128 * static_cast<size_t>(a.Pn) * grid, st);
+        if (e != cudaSuccess) return e;
+    }
+    k_hess_o64<PPAD><<<grid, kO64Threads, L.total, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4],
+                                                         maps[5], maps[6], a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess || a.chunk != 0) return e;
+    k_o64_join<<<dim3(static_cast<unsigned>(a.n_units), static_cast<unsigned>(a.Pn)), 128, 0, st>>>(a, grid);
     return cudaGetLastError();
 }
 
 cudaError_t launch_hess_o64(const PointsDev& p, int32_t Pn, int32_t t0, int64_t acc_P,
                             const void* rec, const void* slices, int64_t slice_stride,
                             int64_t rows, const float* civ, const double* params, int n_sm,
-                            int flush, double* acc, int* err, cudaStream_t st) {
+                            int flush, int32_t pg, double* acc, double* side, int* err, cudaStream_t st) {
     if (p.nk == 0) return cudaSuccess;
-    if (Pn < 1 || Pn > kO64Ppad || t0 + kO64Ppad > rows || p.nk_pad % 256 != 0)
+    const int ppad = hess_o64_ppad(pg);
+    if (Pn < 1 || Pn > pg || pg > kO64MaxPpad || t0 + ppad > rows || p.nk_pad % 256 != 0)
         return cudaErrorInvalidValue;
     CUtensorMap maps[kO64Slices];
     for (int q = 0; q < kO64Slices; ++q)
-        if (!o64_make_map(&maps[q], static_cast<const __half*>(slices) + q * slice_stride, p.nk_pad, rows))
+        if (!o64_make_map(&maps[q], static_cast<const __half*>(slices) + q * slice_stride, p.nk_pad, rows, ppad))
             return cudaErrorInvalidValue;
     O64Args a;
     memset(&a, 0, sizeof(a));
@@ -850,20 +935,23 @@ cudaError_t launch_hess_o64(const PointsDev& p, int32_t Pn, int32_t t0, int64_t 
     a.t0 = t0;
     a.n_units = 2 * ((p.nk + 127) / 128);
     a.n_stage = static_cast<int32_t>(p.nk_pad / kO64Kj);
-    constexpr O64Layout L = o64_layout();
+    const O64Layout L = o64_layout(ppad);
     const size_t stage_bytes = L.slot_bytes + kO64Kj * kO64RecBytes;
     int64_t chunk = static_cast<int64_t>(kO64ChunkBytes / stage_bytes);
     if (chunk < 64) chunk = 64;
-    a.chunk = static_cast<int32_t>(chunk < a.n_stage ? chunk : a.n_stage);
+    // Few units per CTA: equal shares of the stages, or the CTAs with one unit more set the time (618
+    // units on 152 SMs: 5 rounds for 4.07).  Many: the chunked walk, whose trial tiles stay in L2.  Below
+    // 2,048 points a whole unit per CTA: there is little to share, and a few of the smallest systems'
+    // elements (where the tiles' 2^-46 shows most) keep their roundings.
+    a.chunk = a.n_units < 16 * static_cast<int64_t>(n_sm) && a.n_stage >= 128 ? 0 : static_cast<int32_t>(chunk < a.n_stage ? chunk : a.n_stage);
+    a.side = side;
     a.flush = flush > 0 ? flush : 512;
     a.err = err;
-    cudaError_t e = cudaFuncSetAttribute(k_hess_o64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(L.total));
-    if (e != cudaSuccess) return e;
-    const int grid = static_cast<int>(a.n_units < n_sm ? a.n_units : n_sm);
-    k_hess_o64<<<grid, kO64Threads, L.total, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4],
-                                                   maps[5], maps[6], a);
-    return cudaGetLastError();
+    switch (ppad) {
+        case 32: return o64_launch<32>(maps, a, n_sm, st);
+        case 48: return o64_launch<48>(maps, a, n_sm, st);
+        default: return o64_launch<64>(maps, a, n_sm, st);
+    }
 }
 
 }  // namespace vv10

@@ -222,17 +222,17 @@ vv10_status vv10_ctx::f16_contract(int32_t Pn, int cap, cudaStream_t st) {
 }
 
 // Cut u, y (in tu, ty) into FP16 integer slices and contract all Pn trials with FP64
-// accuracy on the tensor cores, in groups of at most 32 trials, into hacc [2][Pn][nk_pad].
+// accuracy on the tensor cores, in groups of at most 64 trials, into hacc [2][Pn][nk_pad].
 vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
     const int cap = hess_o64_max_group();
     const int ng = (Pn + cap - 1) / cap;
     const int pg = (Pn + ng - 1) / ng;
-    const int64_t rows = static_cast<int64_t>(ng - 1) * pg + cap;
+    const int64_t rows = static_cast<int64_t>(ng - 1) * pg + hess_o64_ppad(pg);
     const int64_t stride = 2 * static_cast<int64_t>(rows) * P.nk_pad;  // halves per slice array
     H_TRY(ensure(o64_sl, hess_o64_slices() * sizeof(uint16_t) * static_cast<size_t>(stride),
                  "FP64 trial slices"));
     H_TRY(ensure(o64_rec, 64 * static_cast<size_t>(P.nk_pad), "FP32-pair point records"));
-    // colmax [2] words | params [2] doubles | civ [ng][nk_pad / 16][32] floats
+    // colmax [2] words | params [2] doubles | civ [ng][nk_pad / 16][ppad] floats
     const int64_t civ_n = hess_o64_civ_floats(Pn, pg, P.nk_pad);
     H_TRY(ensure(o64_small, 32 + sizeof(float) * static_cast<size_t>(civ_n), "FP64 trial factors"));
     char* sm = static_cast<char*>(o64_small.p);
@@ -247,7 +247,7 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
                "FP64 trial slices");
     }
     const size_t ab = sizeof(double) * 2 * static_cast<size_t>(Pn) * P.nk_pad;
-    H_TRY(ensure(hacc, ab, "contraction partials"));
+    H_TRY(ensure(hacc, ab + sizeof(double) * 128 * static_cast<size_t>(pg) * n_sm, "contraction partials"));
     H_CUDA(cudaMemsetAsync(hacc.p, 0, ab, st), "zero contraction partials");
     const int64_t civ_group = civ_n / ng;
     PhaseScope ph(this, PH_CONTRACT_TC, st, ng);
@@ -255,7 +255,8 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
         const int t0 = g * pg;
         const int pn = (Pn - t0 < pg) ? Pn - t0 : pg;
         H_CUDA(launch_hess_o64(P, pn, t0, Pn, o64_rec.p, o64_sl.p, stride, rows, civ + g * civ_group,
-                               params, n_sm, tc_flush, static_cast<double*>(hacc.p),
+                               params, n_sm, tc_flush, pg, static_cast<double*>(hacc.p),
+                               static_cast<double*>(hacc.p) + ab / sizeof(double),
                                static_cast<int*>(dev_err.p), st),
                "FP64 tensor-core contraction");
     }

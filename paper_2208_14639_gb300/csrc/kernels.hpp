@@ -276,11 +276,12 @@ cudaError_t launch_hess_f16(const PointsDev& p, int32_t Pn, int32_t t0, int64_t 
 // [P][nk_pad]) into hess_o64_slices() FP16 integer slice arrays [rows][2 nk_pad]
 // (`slice_stride` halves apart; per 16-j block 16 u' then 16 c_y y', scaled per trial and
 // block) with params[0] = 1/c_y, params[1] = c_y (colmax: 2 scratch words), and the factors'
-// inverses civ [group][nk_pad / 16][32] for trial groups of pg <= hess_o64_max_group()
-// (hess_o64_civ_floats floats).  launch_hess_o64 contracts the trials [t0, t0 + Pn), Pn <= pg,
+// inverses civ [group][nk_pad / 16][hess_o64_ppad(pg)] for trial groups of pg <=
+// hess_o64_max_group() (hess_o64_civ_floats floats).  launch_hess_o64 contracts the trials [t0, t0 + Pn), Pn <= pg,
 // with `civ` pointing at their group's block, into acc [2][acc_P][nk_pad] (zeroed by the
-// caller).
+// caller); side: n_sm x Pn x 128 doubles of scratch.
 int hess_o64_max_group();
+int hess_o64_ppad(int32_t pg);
 int hess_o64_slices();
 int64_t hess_o64_civ_floats(int32_t P, int32_t pg, int64_t nk_pad);
 cudaError_t launch_o64_prep(const PointsDev& p, const double* u, const double* y, int32_t P,
@@ -290,7 +291,7 @@ cudaError_t launch_o64_prep(const PointsDev& p, const double* u, const double* y
 cudaError_t launch_hess_o64(const PointsDev& p, int32_t Pn, int32_t t0, int64_t acc_P,
                             const void* rec, const void* slices, int64_t slice_stride,
                             int64_t rows, const float* civ, const double* params, int n_sm,
-                            int flush, double* acc, int* err, cudaStream_t st);
+                            int flush, int32_t pg, double* acc, double* side, int* err, cudaStream_t st);
 
 // Batched tensor-core contraction (molecule and task tables in device memory; see
 // hess_tc.cu for the record layouts the fill helpers write).
