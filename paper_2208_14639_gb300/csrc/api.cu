@@ -403,6 +403,14 @@ vv10_status vv10_ctx::run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_s
     const int nq = pair_mode_nq(mode);
     const int phase = (mode == MODE_EUW || mode == MODE_EUWABC || mode == MODE_EUWABCG) ? PH_PAIR_EUW
                       : (mode == MODE_ABC ? PH_PAIR_ABC : PH_PAIR_GRAD);
+    if (!debug_stall && fp64 && pairsum_rows64_applies(P.nk) && !pairsum_fixed(mode, fp64)) {
+        const int ns = pairsum_rows64_splits(P.nk_pad);
+        VV10_TRY(ensure(part, sizeof(double) * nq * static_cast<size_t>(ns) * P.nk_pad, "pair-sum partials"));
+        PhaseScope ph(this, phase, st, 1);
+        VV10_CUDA(this, launch_pairsum_rows64(P, mode, static_cast<double*>(part.p), st), "pair-sum kernel");
+        *n_split_out = ns;
+        return VV10_OK;
+    }
     if (!debug_stall && pairsum_sym(mode, fp64)) {
         VV10_TRY(ensure(part, sizeof(double) * nq * static_cast<size_t>(P.nk_pad), "pair sums"));
         int n_launch = 0;
@@ -435,14 +443,18 @@ vv10_status vv10_ctx::run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_s
     return VV10_OK;
 }
 
-// Whether a mode's sums run over unordered pairs: at the sizes where that is faster, unless
-// vv10_set_tiles fixed a shape of the row-by-row kernel.
-bool vv10_ctx::pairsum_sym(int mode, bool fp64) const {
+// Whether vv10_set_tiles fixed a shape of the row-by-row kernel for a mode's sums.
+bool vv10_ctx::pairsum_fixed(int mode, bool fp64) const {
     const TileOverride& o = overrides[mode + kPairModes * (fp64 ? 1 : 0)];
     const TileOverride& e = overrides[MODE_EUW + kPairModes * (fp64 ? 1 : 0)];
     const bool fused = (mode == MODE_EUWABC || mode == MODE_EUWABCG);
     const TileOverride* use = o.active ? &o : ((fused && e.active) ? &e : nullptr);
-    return !(use && use->manual) && pairsum_sym_applies(P.nk, fp64);
+    return use && use->manual;
+}
+
+// Whether a mode's sums run over unordered pairs: at the sizes where that is faster.
+bool vv10_ctx::pairsum_sym(int mode, bool fp64) const {
+    return !pairsum_fixed(mode, fp64) && pairsum_sym_applies(P.nk, fp64);
 }
 
 // Tiles of a pair-sum mode: its own override (fixed or tuned), else (fused mode) the

@@ -129,7 +129,8 @@ vv10_status vv10_ctx::tune_pairsum(int mode, bool fp64, cudaStream_t st, bool fo
     }
     float best = 3.0e38f;
     int best_r = fp64 ? 1 : 2, best_s = 0;
-    if (pairsum_sym(mode, fp64)) {  // no shape to choose: the unordered-pair kernel runs
+    // no shape to choose where the unordered-pair or the small FP64 kernel runs
+    if (pairsum_sym(mode, fp64) || (fp64 && pairsum_rows64_applies(P.nk))) {
         o = TileOverride{true, false, mode, fp64, best_r, pairsum_default_split(P, mode, fp64, best_r, n_sm), nb};
         return VV10_OK;
     }

@@ -28,6 +28,7 @@ __global__ void k_grad_epilogue(PointsDev P, const double* __restrict__ part, in
     const int64_t i = P.orig[p];
     for (int d = 0; d < 3; ++d) {
         double s = 0.0;
+#pragma unroll 8
         for (int k = 0; k < n_split; ++k) s += part[(static_cast<int64_t>(d) * n_split + k) * P.nk_pad + p];
         const double g = c * s;
         gk[3 * p + d] = g;

@@ -155,6 +155,11 @@ cudaError_t launch_pairsum(const PointsDev& p, int mode, bool fp64, const PairLa
                            double* part, int* err, cudaStream_t st);
 int pairsum_default_split(const PointsDev& p, int mode, bool fp64, int rows_per_thread, int n_sm);
 
+// FP64 sums of a small system: part[nq][pairsum_rows64_splits(nk_pad)][nk_pad].
+bool pairsum_rows64_applies(int64_t nk);
+int pairsum_rows64_splits(int64_t nk_pad);
+cudaError_t launch_pairsum_rows64(const PointsDev& p, int mode, double* part, cudaStream_t st);
+
 // The same sums over unordered pairs (pairsum_sym.cu): total[nq][nk_pad] FP64, one split; `work`
 // holds pairsum_sym_work() bytes (n_launch: launches of the pair kernel, each followed
 // by one of its reduction).  pairsum_sym_applies: the

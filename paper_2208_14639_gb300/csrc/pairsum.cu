@@ -69,6 +69,38 @@ k_pairsum(const typename Recs<T>::A* __restrict__ ra, const typename Recs<T>::B*
 
 static inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// FP64 sums of a small system, row by row: a CTA takes 128 rows and kRows64J of the j, so that a few
+// hundred points give a few hundred CTAs (an SM's narrow FP64 pipe is what the CTAs on it queue
+// for).  E/U/W with the epilogues: 757 points 54 us (unordered pairs 113, j tiles of 256 240), 3,547
+// points 577 (692); at 5,378 the unordered pairs are ahead, 1,257 against 1,310.
+constexpr int kRows64J = 32;
+template <int MODE>
+__global__ void __launch_bounds__(128)
+k_pairsum_rows64(const double4* __restrict__ ra, const double4* __restrict__ rb, int64_t nk, int64_t nk_pad,
+                 double* __restrict__ part) {
+    constexpr int NQ = pair_mode_nq(MODE);
+    __shared__ double4 sa[kRows64J], sb[kRows64J];
+    const int64_t j0 = static_cast<int64_t>(blockIdx.y) * kRows64J;
+    if (threadIdx.x < kRows64J) {
+        sa[threadIdx.x] = ra[j0 + threadIdx.x];
+        sb[threadIdx.x] = rb[j0 + threadIdx.x];
+    }
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * 128 + threadIdx.x;  // < nk_pad
+    const double4 a = ra[i], b = rb[i];
+    const Row<double> row{a.x, a.y, a.z, b.x, b.y};
+    double acc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
+    __syncthreads();
+#pragma unroll 4
+    for (int jj = 0; jj < kRows64J; ++jj) pair_accumulate<double, MODE>(row, sa[jj], sb[jj], acc);
+    if (i < nk) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            part[(static_cast<int64_t>(q) * gridDim.y + blockIdx.y) * nk_pad + i] = acc[q];
+    }
+}
+
 // Normalise a requested split count so that every split holds whole tiles.
 static inline void split_geometry(int64_t nk_pad, int req, int64_t& j_per_split, int& n_split) {
     const int64_t ntile = nk_pad / kJTile;
@@ -160,6 +192,23 @@ static cudaError_t launch_mode(const PointsDev& p, bool fp64, const PairLaunch& 
     return launch_t<float, MODE, 1, 256>(p, p.r32a, p.r32b, cfg.n_split, cfg.stall, part, err, st);
 }
 
+// Up to 4,096 points: there the unordered-pair kernel's few warps wait for their own FP64 latency.
+bool pairsum_rows64_applies(int64_t nk) { return nk <= 4096; }
+int pairsum_rows64_splits(int64_t nk_pad) { return static_cast<int>(nk_pad / kRows64J); }
+
+cudaError_t launch_pairsum_rows64(const PointsDev& p, int mode, double* part, cudaStream_t st) {
+    if (p.nk == 0) return cudaSuccess;
+    const dim3 grid(static_cast<unsigned>(cdiv(p.nk, 128)), static_cast<unsigned>(pairsum_rows64_splits(p.nk_pad)));
+    switch (mode) {
+        case MODE_EUW: k_pairsum_rows64<MODE_EUW><<<grid, 128, 0, st>>>(p.r64a, p.r64b, p.nk, p.nk_pad, part); break;
+        case MODE_ABC: k_pairsum_rows64<MODE_ABC><<<grid, 128, 0, st>>>(p.r64a, p.r64b, p.nk, p.nk_pad, part); break;
+        case MODE_GRAD: k_pairsum_rows64<MODE_GRAD><<<grid, 128, 0, st>>>(p.r64a, p.r64b, p.nk, p.nk_pad, part); break;
+        case MODE_EUWABC: k_pairsum_rows64<MODE_EUWABC><<<grid, 128, 0, st>>>(p.r64a, p.r64b, p.nk, p.nk_pad, part); break;
+        default: k_pairsum_rows64<MODE_EUWABCG><<<grid, 128, 0, st>>>(p.r64a, p.r64b, p.nk, p.nk_pad, part); break;
+    }
+    return cudaGetLastError();
+}
+
 int pairsum_split_count(int64_t nk_pad, int req) {
     int64_t jps;
     int ns;
@@ -186,6 +235,7 @@ int ep_epilogue_blocks(int64_t nk) { return static_cast<int>(cdiv(nk > 0 ? nk : 
 __device__ __forceinline__ double sum_splits(const double* part, int q, int n_split,
                                              int64_t nk_pad, int64_t p) {
     double s = 0.0;
+#pragma unroll 8
     for (int k = 0; k < n_split; ++k) s += part[(static_cast<int64_t>(q) * n_split + k) * nk_pad + p];
     return s;
 }

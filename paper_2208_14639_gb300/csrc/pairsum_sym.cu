@@ -440,10 +440,10 @@ k_sym_reduce(SymGeom G, const double* __restrict__ rowpart, const T* __restrict_
     const int J = static_cast<int>(p / TS), e = static_cast<int>(p % TS);
     T hi = T(0), lo = T(0);  // column sums
     double sum = add ? total[q * G.nkp + p] : 0.0;
-    const int64_t off = G.d1 - G.d0, w1 = G.owner((J + 1) * off - 1);
-    for (int64_t w = G.owner(J * off); w <= w1; ++w) {
-        const double* r = rowpart + (w * G.max_seg + J - G.first(w) / off) * (NQ * TS * row_parts<T>()) +
-                          (q * R + e % R) * 32 + e / R;
+    const int64_t off = G.d1 - G.d0, w0 = G.owner(J * off), w1 = G.owner((J + 1) * off - 1);
+    int64_t seg = J - G.first(w0) / off;  // the first share may have begun in an earlier tile
+    for (int64_t w = w0; w <= w1; ++w, seg = 0) {
+        const double* r = rowpart + (w * G.max_seg + seg) * (NQ * TS * row_parts<T>()) + (q * R + e % R) * 32 + e / R;
         if constexpr (sizeof(T) == 8) {
             acc_exact(hi, lo, r[0]);
             lo += r[NQ * TS];
@@ -603,8 +603,8 @@ cudaError_t sym_any(const PointsDev* p, int64_t nkp, int mode, bool fp64, int n_
 
 // FP32: a tile pair is one warp's work, so below some thirty tiles the warps are too few (7,211
 // points E/U/W 0.114 ms against 0.108 row by row, 11,932 points 0.151 against 0.19).  FP64: the
-// tiles shrink with the system (702 points 0.08 ms against 0.24); up to 128 points are one row
-// tile's work either way.
+// tiles shrink with the system; the smallest systems take pairsum.cu's small FP64 kernel before
+// this rule is asked.
 bool pairsum_sym_applies(int64_t nk, bool fp64) { return nk > (fp64 ? 128 : 8192); }
 
 size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, int* n_launch) {

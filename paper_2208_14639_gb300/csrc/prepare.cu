@@ -55,6 +55,7 @@ __device__ __forceinline__ void prep_count_block(int64_t n, const double* __rest
     const int64_t base = blk * kPB;
     const int64_t end = min(n, base + kPB);
     int bad = 0;
+#pragma unroll 4
     for (int64_t i = base + threadIdx.x; i < end; i += blockDim.x) {
         const double x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
         if (!finite3(x, y, z) || !isfinite(w[i]) || isnan(rho[i]) ||
@@ -140,11 +141,17 @@ __device__ __forceinline__ void prep_scan_block(const int32_t* __restrict__ hist
         offs[k] = run;
         run += hist[k];
     }
-    if (t < 6) {
-        double v = (t < 3) ? INFINITY : -INFINITY;
-        for (int b = 0; b < nblk; ++b)
-            v = (t < 3) ? fmin(v, bbox_part[b * 6 + t]) : fmax(v, bbox_part[b * 6 + t]);
-        shb[t] = v;
+    if (t < 6 * 32) {  // a warp per bound
+        const int d = t >> 5;
+        double v = (d < 3) ? INFINITY : -INFINITY;
+        for (int b = t & 31; b < nblk; b += 32)
+            v = (d < 3) ? fmin(v, bbox_part[b * 6 + d]) : fmax(v, bbox_part[b * 6 + d]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v, o);
+            v = (d < 3) ? fmin(v, u) : fmax(v, u);
+        }
+        if ((t & 31) == 0) shb[d] = v;
     }
     __syncthreads();  // offs complete, bbox reduced
     const int64_t nk = offs[static_cast<int64_t>(n_keys - 1) * nblk];
@@ -187,8 +194,24 @@ __device__ __forceinline__ void prep_scatter_block(int64_t n, const double* __re
         sh_key[q] = point_key(base + q, rho, atom, n_atom, rho_cut, n_keys, keep);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {  // caller order within the block -> stable
-        for (int q = 0; q < cnt; ++q) sh_pos[q] = sh_cnt[sh_key[q]]++;
+    // One warp takes the points in caller order, 32 at a time; equal keys are ranked by lane, so the
+    // order within a key is the caller's.  (One thread taking them one by one: 39 us a launch, at any
+    // size; this 4.)
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        for (int q0 = 0; q0 < cnt; q0 += 32) {
+            const int q = q0 + lane;
+            const int key = q < cnt ? sh_key[q] : -1;
+            const unsigned same = __match_any_sync(0xffffffffu, key);
+            const int rank = __popc(same & ((1u << lane) - 1u));
+            const int64_t first = key >= 0 ? sh_cnt[key] : 0;
+            __syncwarp();
+            if (key >= 0) {
+                sh_pos[q] = first + rank;
+                if (rank == 0) sh_cnt[key] = first + __popc(same);
+            }
+            __syncwarp();
+        }
     }
     __syncthreads();
     for (int q = threadIdx.x; q < cnt; q += blockDim.x)
@@ -349,8 +372,10 @@ cudaError_t launch_prepare_scatter(int64_t n, const double* xyz, const double* w
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (nk_pad > 0) {
-        const int g = static_cast<int>((nk_pad + 255) / 256);
-        k_prep_points<<<g, 256, 0, st>>>(nk, nk_pad, orig, xyz, w, rho, grad, atom, b, C,
+        // two warps a CTA: some 350 FP64 operations a point, which few CTAs would queue on few SMs'
+        // FP64 pipes (936 points: 17 us in CTAs of 256)
+        const int g = static_cast<int>((nk_pad + 63) / 64);
+        k_prep_points<<<g, 64, 0, st>>>(nk, nk_pad, orig, xyz, w, rho, grad, atom, b, C,
                                          s.center, atom_k, soa, r64a, r64b, r32a, r32b, r32p);
         e = cudaGetLastError();
     }

@@ -212,6 +212,7 @@ struct vv10_ctx {
     vv10_status require_prepared();
     vv10::PointsDev points() const;
     vv10::TileChoice tiles_for(int mode, bool fp64) const;
+    bool pairsum_fixed(int mode, bool fp64) const;
     bool pairsum_sym(int mode, bool fp64) const;
     vv10_status run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_split_out);
     // autotuner (autotune.cu)

@@ -1,5 +1,6 @@
-"""The unordered-pair sums (pairsum_sym.cu) against the row-by-row kernel (fixed with
-vv10_set_tiles), whose values the oracle tests pin: every mode, at the edges of their tiles.
+"""The unordered-pair sums (pairsum_sym.cu) and the small FP64 kernel (pairsum.cu) against the
+row-by-row kernel (fixed with vv10_set_tiles), whose values the oracle tests pin: every mode, at
+the edges of their tiles and of their ranges.
 
 Both form the same FP32 sum over each 256-point tile and add the tiles in FP64 (rows) or
 double-FP32 (columns: 2^-47 per tile at most), so the mixed results may differ by a few hundred
@@ -45,9 +46,10 @@ def results(g, prec, classic, dev):
     return [torch.as_tensor(x, dtype=torch.float64).cpu() for x in out]
 
 
-# FP64: one tile, fewer and more rows per lane, odd and even tile counts (the half turn), one
-# point past a tile; mixed: the smallest size of the rule, and odd and even tile counts.
-@pytest.mark.parametrize("prec,n", [(FP64, n) for n in (129, 255, 256, 257, 700, 1024, 1025, 2305, 6000)] +
+# FP64: one tile and one point past a tile, both sides of the rule at 4,096, fewer and more rows per
+# lane, odd and even tile counts (the half turn); mixed: the smallest size of the rule, and odd and
+# even tile counts.
+@pytest.mark.parametrize("prec,n", [(FP64, n) for n in (1, 129, 255, 256, 257, 1025, 4096, 4097, 4352, 4353, 4609, 6000)] +
                          [(MIXED, n) for n in (8193, 8448, 8449, 8705, 9900)])
 def test_unordered_pairs_match_rows(dev, prec, n):
     g = synth.random_points(n, seed=n, n_atom=3)
