@@ -897,13 +897,19 @@ vv10_status vv10_weight_response(vv10_handle h, vv10_precision prec, int32_t P,
         weight_tc_groups(P, &ng, &ppad);
         const int32_t rows = ng * ppad;
         const size_t nsplit = static_cast<size_t>(rows) * static_cast<size_t>(Pd.nk_pad);
-        VV10_TRY(h->ensure(h->wsplit, 2 * sizeof(float) * nsplit, "weight direction split"));
+        // nsplit is a multiple of 32 x 64: the side outputs after the split stay aligned
+        const size_t side_n = weight_tc_side(Pd.nk_pad, ppad, h->n_sm);
+        bool shares = side_n > 0 && h->ensure(h->wsplit, 2 * sizeof(float) * nsplit + sizeof(double) * side_n,
+                                              "weight direction split") == VV10_OK;
+        if (!shares) VV10_TRY(h->ensure(h->wsplit, 2 * sizeof(float) * nsplit, "weight direction split"));
+        h->set_error("");
         float* yh = static_cast<float*>(h->wsplit.p);
-        PhaseScope ph(h, PH_WEIGHT_RESPONSE, st, 3);
+        double* side = shares ? reinterpret_cast<double*>(yh + 2 * nsplit) : nullptr;
+        PhaseScope ph(h, PH_WEIGHT_RESPONSE, st, side ? 4 : 3);
         VV10_CUDA(h, launch_weight_dirs(Pd, P, w_t, yk, st), "weight directions");
         VV10_CUDA(h, launch_weight_split(yk, P, rows, Pd.nk_pad, yh, yh + nsplit, st),
                   "weight direction split");
-        VV10_CUDA(h, launch_weight_tc(Pd, P, yh, yh + nsplit, rows, E_t, U_t, W_t, h->n_sm,
+        VV10_CUDA(h, launch_weight_tc(Pd, P, yh, yh + nsplit, rows, E_t, U_t, W_t, h->n_sm, side,
                                       static_cast<int*>(h->dev_err.p), st),
                   "weight-derivative sums (tensor cores)");
         return VV10_OK;

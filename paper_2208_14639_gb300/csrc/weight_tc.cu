@@ -5,8 +5,8 @@
 // three N x N kernel matrices times the N x P direction matrix, split-TF32 (hi*hi + hi*lo +
 // lo*hi) on tcgen05.
 //
-// Work unit ("task"): 128 rows i x one group of at most 64 directions (N of the MMA) x every
-// j.  A persistent CTA walks its tasks; per stage of 16 j:
+// Task: 128 rows i x one group of at most 64 directions (N of the MMA) x every j.  A persistent
+// CTA walks its share of them; per stage of 16 j:
 //   * 16 generator warps (4 per row quadrant, 4 j each) evaluate K1, K2, K3 for their row in
 //     FP32 and split them into TF32 hi/lo: the three hi tiles go to tensor memory (their MMAs
 //     read no shared memory for A), the three lo tiles to shared memory in the
@@ -19,7 +19,12 @@
 //     and commits the stage once;
 //   * the generator warps drain the finished stage's accumulators into FP32 registers,
 //     release the ring slot, and every `flush` stages add the registers into the FP64
-//     outputs (each task's rows and directions are owned by one CTA: no atomics).
+//     outputs.
+// The pieces of `flush` stages of all tasks are dealt to the CTAs in equal contiguous shares: whole
+// tasks of a few rounds leave the chip idle in the last (39,542 kept points, 36 directions: 309 tasks
+// on 152 SMs, three rounds for 2.03: 7.45 -> 5.60 ms).  A share that begins inside a task writes that
+// part to its own side output, added in CTA order at the end (no atomics); the FP32 sums end at the
+// same stages, only the order of FP64 additions can differ.
 // As in the Hessian contraction, each TMEM accumulation run is one stage with the hi*lo and
 // lo*hi products first and the hi*hi products last (the tensor core truncates).
 #include <cstring>
@@ -41,6 +46,7 @@ constexpr int kWtThreads = (kWtGenWarps + 2) * 32;
 constexpr int kWtRing = 4;                      // stages of direction tiles in flight
 constexpr int kWtKinds = 3;                     // E, U, W
 constexpr int kWtMaxPpad = 64;
+constexpr int kWtFlush = 512;                   // stages per FP64 flush
 constexpr uint32_t kWtTmemCols = 512;
 constexpr uint32_t kWtATile = 128u * 64u;       // one 128 x 16 tf32 operand tile (bytes)
 constexpr uint32_t kWtABuf = kWtKinds * kWtATile;  // the lo parts of the three kernel tiles
@@ -76,7 +82,34 @@ struct WtArgs {
     int32_t n_groups;     // direction groups of Ppad
     int64_t n_tasks;      // row tiles x groups
     int flush;            // stages per FP64 flush
+    double* side;         // [CTA][kind][Ppad][128] output of a share's first task if it is a begun one
     int* err;
+    // Shares: the pieces of `flush` stages (what one FP64 flush sums) in the order (task, piece) are
+    // dealt evenly; without `side` a piece is a whole task.
+    __host__ __device__ int n_stage() const { return static_cast<int>(nk_pad / kWtKj); }
+    __host__ __device__ int pieces() const { return side ? (n_stage() + flush - 1) / flush : 1; }  // of a task
+    __host__ __device__ int64_t first(int64_t cta, int64_t grid) const { return cta * (n_tasks * pieces()) / grid; }
+};
+
+// The segments of a CTA's share: task q, stages s0 .. s1 - 1 (begun: not the task's first ones).
+struct WtWalk {
+    int64_t p, p1, q;
+    int s0, s1;
+    bool begun;
+    __device__ __forceinline__ explicit WtWalk(const WtArgs& a)
+        : p(a.first(blockIdx.x, gridDim.x)), p1(a.first(blockIdx.x + 1, gridDim.x)), q(0), s0(0), s1(0), begun(false) {}
+    __device__ __forceinline__ bool next(const WtArgs& a) {
+        if (p >= p1) return false;
+        const int np = a.pieces();
+        q = p / np;
+        const int k = static_cast<int>(p - q * np);
+        const int k1 = static_cast<int>(min(static_cast<int64_t>(np), k + (p1 - p)));
+        p += k1 - k;
+        s0 = k * a.flush;
+        s1 = (k1 == np) ? a.n_stage() : k1 * a.flush;
+        begun = k > 0;
+        return true;
+    }
 };
 
 __device__ __forceinline__ bool wt_wait(uint64_t* bar, uint32_t parity, int* err,
@@ -148,7 +181,6 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kWtRing + 6);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_stage = static_cast<int>(args.nk_pad / kWtKj);
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < kWtRing; ++b) {
@@ -178,9 +210,9 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             uint32_t ph = 0;
             int64_t issued = 0;
             bool ok = true;
-            for (int64_t q = blockIdx.x; q < args.n_tasks && ok; q += gridDim.x) {
-                const int t0 = static_cast<int>(q % args.n_groups) * PPAD;
-                for (int s = 0; s < n_stage; ++s) {
+            for (WtWalk w(args); ok && w.next(args);) {
+                const int t0 = static_cast<int>(w.q % args.n_groups) * PPAD;
+                for (int s = w.s0; s < w.s1; ++s) {
                     if (!wt_wait(&b_empty[slot], ph ^ 1u, args.err, abort_flag)) {
                         ok = false;
                         break;
@@ -211,8 +243,8 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             int slot = 0, ab = 0;
             uint32_t ph = 0, aph = 0;
             bool ok = true, issued_any = false;
-            for (int64_t q = blockIdx.x; q < args.n_tasks && ok; q += gridDim.x) {
-                for (int s = 0; s < n_stage; ++s) {
+            for (WtWalk w(args); ok && w.next(args);) {
+                for (int s = w.s0; s < w.s1; ++s) {
                     if (!wt_wait(&a_full[ab], aph, args.err, abort_flag) ||
                         !wt_wait(&b_full[slot], ph, args.err, abort_flag)) {
                         ok = false;
@@ -291,7 +323,7 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             tc::fence_before();
             return true;
         };
-        auto flush = [&](int t0, int64_t i) {
+        auto flush = [&](int t0, int64_t i, bool begun, bool fresh) {
             const bool row_ok = i < args.nk;
             const int64_t oi = row_ok ? args.orig[i] : 0;
 #pragma unroll
@@ -302,7 +334,9 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
                     const int t = t0 + part * PQ + c;
                     if (o && row_ok && t < args.P) {
                         const double v = static_cast<double>(acc[k][c]);
-                        o[static_cast<int64_t>(t) * args.n + oi] += (k == 0) ? v : -v;
+                        double* x = begun ? args.side + ((static_cast<int64_t>(blockIdx.x) * kWtKinds + k) * PPAD + t - t0) * 128 + r
+                                          : o + static_cast<int64_t>(t) * args.n + oi;
+                        *x = (fresh ? 0.0 : *x) + ((k == 0) ? v : -v);
                     }
                     acc[k][c] = 0.0f;
                 }
@@ -313,9 +347,9 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
         uint32_t ph = 0, aph = 0;
         int pslot = 0, dbuf = 0;
         uint32_t dph = 0;
-        for (int64_t q = blockIdx.x; q < args.n_tasks && ok; q += gridDim.x) {
-            const int64_t row_tile = q / args.n_groups;
-            const int t0 = static_cast<int>(q % args.n_groups) * PPAD;
+        for (WtWalk w(args); ok && w.next(args);) {
+            const int64_t row_tile = w.q / args.n_groups;
+            const int t0 = static_cast<int>(w.q % args.n_groups) * PPAD;
             const int64_t i = row_tile * 128 + r;
             float xi = 0.f, yi = 0.f, zi = 0.f, oi = 1.f, ki = 1.f;
             if (i < args.nk) {
@@ -326,7 +360,8 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             const float2 X = make_float2(xi, xi), Y = make_float2(yi, yi), Z = make_float2(zi, zi);
             const float2 O = make_float2(oi, oi), K = make_float2(ki, ki);
             int until_flush = args.flush;
-            for (int s = 0; s < n_stage; ++s) {
+            bool fresh = w.begun;  // the side output holds nothing yet
+            for (int s = w.s0; s < w.s1; ++s) {
                 // operand buffer ab is free once the MMAs of the stage two back are done
                 bool got = wt_wait(&b_full[slot], ph, args.err, abort_flag);
                 got = got && wt_wait(&mma_done[ab], aph ^ 1u, args.err, abort_flag);
@@ -364,14 +399,15 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&a_full[ab]);
                 // drain the previous stage while this stage's MMAs run
-                if (s > 0) {
+                if (s > w.s0) {
                     if (!drain(dbuf, dph)) {
                         ok = false;
                         break;
                     }
                     if (lane == 0) mbar_arrive(&b_empty[pslot]);
                     if (--until_flush == 0) {
-                        flush(t0, i);
+                        flush(t0, i, w.begun, fresh);
+                        fresh = false;
                         until_flush = args.flush;
                     }
                 }
@@ -391,7 +427,7 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
                 break;
             }
             if (lane == 0) mbar_arrive(&b_empty[pslot]);
-            flush(t0, i);
+            flush(t0, i, w.begun, fresh);
         }
         tc::wait_st();  // nothing of ours is in flight to or from TMEM on any exit path
         tc::wait_ld();
@@ -403,6 +439,30 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
         tc::fence_after();
         tc::tmem_dealloc(tmem, kWtTmemCols);
     }
+}
+
+// Adds the side outputs of the CTAs whose shares began inside a task to its outputs, in CTA order.
+// Block = (task, direction of the group), thread = row.
+__global__ void __launch_bounds__(128) k_wresp_join(WtArgs a, int32_t ppad, int32_t grid) {
+    const int64_t q = blockIdx.x, i = (q / a.n_groups) * 128 + threadIdx.x;
+    const int t = static_cast<int>(q % a.n_groups) * ppad + static_cast<int>(blockIdx.y);
+    if (i >= a.nk || t >= a.P) return;
+    const int np = a.pieces();
+    const int64_t b = q * np;
+    double v[kWtKinds] = {0.0, 0.0, 0.0};
+    bool any = false;
+    // shares with b < first(c) < b + np (first(c) = floor(c all / grid))
+    for (int64_t c = (b * grid) / (a.n_tasks * np); c < grid; ++c) {
+        const int64_t f = a.first(c, grid);
+        if (f <= b) continue;
+        if (f >= b + np) break;
+        any = true;
+        for (int k = 0; k < kWtKinds; ++k)
+            if (a.out[k]) v[k] += a.side[((c * kWtKinds + k) * ppad + blockIdx.y) * 128 + threadIdx.x];
+    }
+    if (!any) return;
+    for (int k = 0; k < kWtKinds; ++k)
+        if (a.out[k]) a.out[k][static_cast<int64_t>(t) * a.n + a.orig[i]] += v[k];
 }
 
 // y (Pn x nk_pad FP64, -3/2 rho v) -> TF32 hi and FP32 lo, rows x nk_pad (rows >= Pn are zero).
@@ -424,9 +484,12 @@ cudaError_t launch_wt(const CUtensorMap* maps, const WtArgs& a, int n_sm, cudaSt
     cudaError_t e = cudaFuncSetAttribute(k_wresp_tc<PQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L.total));
     if (e != cudaSuccess) return e;
-    const int grid = static_cast<int>(a.n_tasks < n_sm ? a.n_tasks : n_sm);
+    const int64_t all = a.n_tasks * a.pieces();
+    const int grid = static_cast<int>(all < n_sm ? all : n_sm);
     if (grid <= 0) return cudaSuccess;
     k_wresp_tc<PQ><<<grid, kWtThreads, L.total, st>>>(maps[0], maps[1], a);
+    if ((e = cudaGetLastError()) != cudaSuccess || a.pieces() == 1) return e;
+    k_wresp_join<<<dim3(static_cast<unsigned>(a.n_tasks), 4 * PQ), 128, 0, st>>>(a, 4 * PQ, grid);
     return cudaGetLastError();
 }
 
@@ -448,8 +511,14 @@ cudaError_t launch_weight_split(const double* yk, int32_t Pn, int32_t rows, int6
     return cudaGetLastError();
 }
 
+// Doubles of `side` for equal shares of the stages; 0 where a task is one piece, and whole tasks are dealt.
+// (Whole tasks at 39,542 kept points, 36 directions: 309 on 152 SMs, three rounds for 2.03.)
+size_t weight_tc_side(int64_t nk_pad, int ppad, int n_sm) {
+    return nk_pad > kWtFlush * kWtKj ? static_cast<size_t>(n_sm) * kWtKinds * static_cast<size_t>(ppad) * 128 : 0;
+}
+
 cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, const float* yl,
-                             int32_t rows, double* E, double* U, double* W, int n_sm, int* err,
+                             int32_t rows, double* E, double* U, double* W, int n_sm, double* side, int* err,
                              cudaStream_t st) {
     if (p.nk == 0 || Pn <= 0) return cudaSuccess;
     int ng = 0, ppad = 0;
@@ -473,7 +542,8 @@ cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, co
     a.P = Pn;
     a.n_groups = ng;
     a.n_tasks = static_cast<int64_t>(ng) * ((p.nk + 127) / 128);
-    a.flush = 512;
+    a.flush = kWtFlush;
+    a.side = side;
     a.err = err;
     return ppad == 32 ? launch_wt<8>(maps, a, n_sm, st) : launch_wt<16>(maps, a, n_sm, st);
 }
