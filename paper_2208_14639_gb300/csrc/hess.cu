@@ -12,6 +12,8 @@
 //   f^{gamma,t}_i = sigma_i sum_j (T3 u_jt + T4 y_jt)    + diagonal terms,
 // a product of a generated N x 2N kernel matrix with a 2N x P trial matrix.  The
 // diagonal terms are the delta_ij / w_i parts of the four printed coefficients.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.hpp"
 #include "tc.cuh"
@@ -93,31 +95,42 @@ cudaError_t launch_trial_prep(const PointsDev& p, int32_t P, const double* rho_t
 // ------------------------------------------------------------------ FP64 SIMT contraction
 constexpr int kHessThreads = 128;
 constexpr int kHessJT = 32;
+constexpr int kHessMaxTrials = 40;  // per CTA
 
-// The four generated kernel values of one pair (FP64).
+// The four generated kernel values of one pair, 31 FP64 operations.  The pipe issues about two a clock and
+// SM and bounds the kernel, so: inv = 1/(g g' s) with recip(), L = g g' inv, G_i G_j = s inv,
+// L + G_i = L + g' s inv, L + G_j = L + g s inv, M = 2 M' (M' = L^2 + s inv), and with q = R^2 inv
+//   -2/3 T1 = inv [1 - A_i (L+G_i) + A_j X],  -2/3 T2 = q X,  X = 2 A_i M' - (L+G_j),
+//   -2/3 T3 = q [2 A_j M' - (L+G_i)],         -2/3 T4 = 2 q R^2 M'.
+// p2, q2 (row) and b.z, b.w (column) hold twice rho a's factors; of the results t1 is twice and t4 half
+// its value above (the trial vector u is halved and f^gamma doubled: powers of two, exact).
+// With the IEEE divide and L, G_i, G_j apart it was about 46.  4-atom CHON, 26,400 points, 12 trials
+// (the response call): 65.8 ms with those tiles and 16 trials a CTA, 49.4 ms with these and 12, of
+// which the pipe's rate at 79 operations a pair is about 47.
 struct Tiles64 {
     double t1, t2, t3, t4;
 };
 __device__ __forceinline__ Tiles64 tiles64(double xi, double yi, double zi, double oi, double ki,
-                                           double pi_, double qi, const double4& a,
+                                           double p2, double q2, const double4& a,
                                            const double4& b) {
     const double dx = xi - a.x, dy = yi - a.y, dz = zi - a.z;
     const double r2 = dx * dx + dy * dy + dz * dz;
     const double g = oi * r2 + ki;
     const double gp = b.x * r2 + b.y;
     const double s = g + gp;
-    const double inv = 1.0 / (g * gp * s);
-    const double phi = -1.5 * inv;
-    const double L = g * gp * inv, Gi = gp * s * inv, Gj = g * s * inv;
-    const double M = 2.0 * (L * L + Gi * Gj);
-    const double Ai = pi_ + qi * r2, Aj = b.z + b.w * r2;
-    const double LGi = L + Gi, LGj = L + Gj;
+    const double ggp = g * gp;
+    const double inv = recip(ggp * s);
+    const double L = ggp * inv, si = s * inv;
+    const double M = fma(L, L, si);
+    const double LGi = fma(gp, si, L), LGj = fma(g, si, L);
+    const double Ai = fma(q2, r2, p2), Aj = fma(b.w, r2, b.z);
+    const double X = fma(Ai, M, -LGj);
+    const double q = r2 * inv;
     Tiles64 T;
-    T.t1 = phi * (1.0 - Ai * LGi - Aj * LGj + Ai * Aj * M);
-    const double rp = r2 * phi;
-    T.t2 = rp * (Ai * M - LGj);
-    T.t3 = rp * (Aj * M - LGi);
-    T.t4 = rp * r2 * M;
+    T.t1 = inv * fma(Aj, X, fma(-Ai, LGi, 2.0));
+    T.t2 = q * X;
+    T.t3 = q * fma(Aj, M, -LGi);
+    T.t4 = q * (r2 * M);
     return T;
 }
 
@@ -136,10 +149,10 @@ k_hess_f64(PointsDev P, int32_t Pn, const double* __restrict__ u, const double* 
     const int64_t jb = static_cast<int64_t>(split) * j_per_split;
     const int64_t je = min(P.nk_pad, jb + j_per_split);
 
-    double xi = 0, yi = 0, zi = 0, oi = 1, ki = 1, pi_ = 0, qi = 0;
+    double xi = 0, yi = 0, zi = 0, oi = 1, ki = 1, p2 = 0, q2 = 0;
     if (i < P.nk) {
         const double4 a = P.r64a[i], b = P.r64b[i];
-        xi = a.x; yi = a.y; zi = a.z; oi = b.x; ki = b.y; pi_ = b.z; qi = b.w;
+        xi = a.x; yi = a.y; zi = a.z; oi = b.x; ki = b.y; p2 = 2.0 * b.z; q2 = 2.0 * b.w;
     }
     double ar[PC], ag[PC];
 #pragma unroll
@@ -148,18 +161,23 @@ k_hess_f64(PointsDev P, int32_t Pn, const double* __restrict__ u, const double* 
     for (int64_t j0 = jb; j0 < je; j0 += kHessJT) {
         __syncthreads();
         if (tid < kHessJT) sA[tid] = P.r64a[j0 + tid];
-        else if (tid < 2 * kHessJT) sB[tid - kHessJT] = P.r64b[j0 + tid - kHessJT];
+        else if (tid < 2 * kHessJT) {
+            double4 b = P.r64b[j0 + tid - kHessJT];
+            b.z *= 2.0;
+            b.w *= 2.0;
+            sB[tid - kHessJT] = b;
+        }
         for (int e = tid; e < PC * kHessJT; e += kHessThreads) {
             const int tt = e / kHessJT, jj = e % kHessJT;
             const int t = t0 + tt;
             const int64_t o = static_cast<int64_t>(t) * P.nk_pad + j0 + jj;
-            su[tt][jj] = (t < Pn) ? u[o] : 0.0;
+            su[tt][jj] = (t < Pn) ? 0.5 * u[o] : 0.0;
             sy[tt][jj] = (t < Pn) ? y[o] : 0.0;
         }
         __syncthreads();
 #pragma unroll 1
         for (int jj = 0; jj < kHessJT; ++jj) {
-            const Tiles64 T = tiles64(xi, yi, zi, oi, ki, pi_, qi, sA[jj], sB[jj]);
+            const Tiles64 T = tiles64(xi, yi, zi, oi, ki, p2, q2, sA[jj], sB[jj]);
 #pragma unroll
             for (int k = 0; k < PC; ++k) {
                 const double uu = su[k][jj], yy = sy[k][jj];
@@ -173,8 +191,8 @@ k_hess_f64(PointsDev P, int32_t Pn, const double* __restrict__ u, const double* 
         for (int k = 0; k < PC; ++k) {
             const int t = t0 + k;
             if (t < Pn) {
-                acc[((static_cast<int64_t>(0) * n_split + split) * Pn + t) * P.nk_pad + i] = ar[k];
-                acc[((static_cast<int64_t>(1) * n_split + split) * Pn + t) * P.nk_pad + i] = ag[k];
+                acc[((static_cast<int64_t>(0) * n_split + split) * Pn + t) * P.nk_pad + i] = -1.5 * ar[k];
+                acc[((static_cast<int64_t>(1) * n_split + split) * Pn + t) * P.nk_pad + i] = -3.0 * ag[k];
             }
         }
     }
@@ -189,14 +207,37 @@ static inline void hess_split_geometry(int64_t nk_pad, int req, int64_t& jps, in
     ns = static_cast<int>(ntile > 0 ? cdiv64(ntile, tps) : 1);
 }
 
+// Trials per CTA: the chunks of at most 40 trials (80 FP64 accumulators a thread; eight warps an SM keep
+// the FP64 pipe busy, so registers are there) that need the fewest operations a pair, 31 + 4 per trial
+// and chunk, in the fewest multiples of 4 (1 and 2 for single directions).  Chunks of 8, 16 or 32 did
+// 64 operations for 12 trials' 48.
+int hess_f64_trials_per_cta(int32_t P) {
+    if (P <= 2) return P < 2 ? 1 : 2;
+    const int32_t chunks = static_cast<int32_t>(cdiv64(P, kHessMaxTrials));
+    return static_cast<int>(cdiv64(cdiv64(P, chunks), 4) * 4);
+}
+
+// j splits: between three CTAs an SM and the bound of the partials (six with up to 16 trials), the
+// number that leaves the least work on the fullest SM.
 int hess_f64_default_split(const PointsDev& p, int32_t P, int pc, int n_sm) {
-    const int64_t ctas = cdiv64(p.nk, kHessThreads) * cdiv64(P, pc);
-    const int64_t target = static_cast<int64_t>(n_sm) * 6;
-    int req = static_cast<int>(cdiv64(target, ctas > 0 ? ctas : 1));
-    int64_t jps;
-    int ns;
-    hess_split_geometry(p.nk_pad, req, jps, ns);
-    return ns;
+    const int64_t rows = cdiv64(p.nk, kHessThreads), ctas = rows * cdiv64(P, pc);
+    if (ctas <= 0) return 1;
+    const int64_t hi = cdiv64(6 * static_cast<int64_t>(n_sm), rows * cdiv64(P, 16));
+    const int64_t lo = std::min(hi, cdiv64(3 * static_cast<int64_t>(n_sm), ctas));
+    int best = 1;
+    int64_t best_work = -1;
+    for (int64_t req = lo; req <= hi; ++req) {
+        int64_t jps;
+        int ns;
+        hess_split_geometry(p.nk_pad, static_cast<int>(req), jps, ns);
+        const int64_t work = cdiv64(ctas * ns, n_sm) * jps;
+        if (best_work < 0 || work < best_work) {
+            best_work = work;
+            best = ns;
+        }
+        if (req > p.nk_pad / kJTile) break;
+    }
+    return best;
 }
 
 cudaError_t launch_hess_f64(const PointsDev& p, int32_t P, const double* u, const double* y,
@@ -206,12 +247,24 @@ cudaError_t launch_hess_f64(const PointsDev& p, int32_t P, const double* u, cons
     int64_t jps;
     int ns;
     hess_split_geometry(p.nk_pad, cfg.n_split, jps, ns);
-    const int pc = cfg.trials_per_cta <= 8 ? 8 : (cfg.trials_per_cta <= 16 ? 16 : 32);
+    const int pc = cfg.trials_per_cta;
     dim3 grid(static_cast<unsigned>(cdiv64(p.nk, kHessThreads)),
               static_cast<unsigned>(cdiv64(P, pc)), static_cast<unsigned>(ns));
-    if (pc == 8) k_hess_f64<8><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc);
-    else if (pc == 16) k_hess_f64<16><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc);
-    else k_hess_f64<32><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc);
+    switch (pc) {
+        case 1: k_hess_f64<1><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 2: k_hess_f64<2><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 4: k_hess_f64<4><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 8: k_hess_f64<8><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 12: k_hess_f64<12><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 16: k_hess_f64<16><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 20: k_hess_f64<20><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 24: k_hess_f64<24><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 28: k_hess_f64<28><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 32: k_hess_f64<32><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 36: k_hess_f64<36><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        case 40: k_hess_f64<40><<<grid, kHessThreads, 0, st>>>(p, P, u, y, jps, acc); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

@@ -16,22 +16,6 @@ using namespace vv10;
         if (s_ != VV10_OK) return s_; \
     } while (0)
 
-// Trials per CTA of the FP64 SIMT contraction: minimise chunks * (pair-generation cost +
-// 4 FMAs per trial), the FP64 operation count per pair.
-int vv10::hess_f64_trials_per_cta(int32_t P) {
-    int best = 8;
-    long best_cost = -1;
-    for (int pc : {8, 16, 32}) {
-        const long chunks = (P + pc - 1) / pc;
-        const long cost = chunks * (45 + 4L * pc);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best = pc;
-        }
-    }
-    return best;
-}
-
 vv10_status vv10_ctx::hessian(vv10_precision prec, int32_t Pn, const double* rho_t,
                               const double* grad_rho_t, double* f_rho_t, double* f_gamma_t,
                               cudaStream_t st) {

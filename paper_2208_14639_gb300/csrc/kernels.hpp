@@ -313,7 +313,7 @@ void hess_tc_fill_mol(void* dst, const float4* r32a, const float4* r32b, const f
 void hess_tc_fill_task(void* dst, int32_t mol, int32_t row_tile, int32_t kind);
 
 struct HessLaunch {
-    int trials_per_cta = 16;  // FP64 SIMT: 8, 16, 32
+    int trials_per_cta = 16;  // FP64 SIMT: 1, 2 or a multiple of 4 up to 40
     int n_split = 1;
 };
 int hess_f64_default_split(const PointsDev& p, int32_t P, int pc, int n_sm);
