@@ -15,8 +15,11 @@
 //     the stage once;
 //   * the generator warps drain the finished stage's accumulator into FP32 registers
 //     (round-to-nearest adds), release the stage's ring slot, and every `flush` stages
-//     add the registers into the FP64 partial output in global memory (each tile's rows
-//     are owned by one CTA: no atomics).
+//     add the registers into the FP64 partial output in global memory.
+// Tiles are dealt to the CTAs whole, in turn, or, where that leaves the chip idle in the last round
+// (shares_pay), in equal contiguous shares of the pieces that one FP64 flush sums; a share that begins
+// inside a tile writes that part to its own side output, added in CTA order at the end (no atomics).
+// The FP32 sums end at the same stages either way.
 // The tensor core accumulates with truncation, so each TMEM accumulation run is kept to
 // one stage, with the hi*lo and lo*hi products first and the four hi*hi products last
 // (bits are lost at the scale of the stage sum only in those four adds); the register and
@@ -81,12 +84,19 @@ struct TcArgs {
     const TcTask* tasks;    // batch: task table, largest molecules first (null: implicit)
     int64_t n_tasks;
     int flush;              // stages per FP64 flush
+    double* side;           // shares: [CTA][kind of a tile][Ppad][128] output of a share's first task if it
+                            // is a begun one; null: whole tasks are dealt
     int* err;
+    // Shares (single system): the pieces of `flush` stages in the order (task, piece) are dealt evenly.
+    __host__ __device__ int n_stage() const { return static_cast<int>(single.nk_pad / kTcKj); }
+    __host__ __device__ int pieces() const { return (n_stage() + flush - 1) / flush; }  // of a task
+    __host__ __device__ int first(int64_t cta, int64_t grid) const {
+        return static_cast<int>(cta * (n_tasks * pieces()) / grid);
+    }
 };
 
 template <int NK>
-__device__ __forceinline__ TcTask tc_task(const TcArgs& a, int64_t q) {
-    if (a.tasks) return a.tasks[q];
+__device__ __forceinline__ TcTask tc_task(int q) {
     TcTask t;
     t.mol = 0;
     t.row_tile = static_cast<int32_t>(NK == 2 ? q : (q >> 1));
@@ -94,6 +104,34 @@ __device__ __forceinline__ TcTask tc_task(const TcArgs& a, int64_t q) {
     t.pad = 0;
     return t;
 }
+
+// The segments of a CTA: task tk, stages s0 .. s1 - 1 (begun: not the task's first ones): whole tasks in
+// turn, or with SHARES its share of the pieces.
+template <int NK, bool SHARES>
+struct TcWalk {
+    int p, p1, s0, s1;
+    bool begun;
+    TcTask tk;
+    __device__ __forceinline__ explicit TcWalk(const TcArgs& a)
+        : p(SHARES ? a.first(blockIdx.x, gridDim.x) : static_cast<int>(blockIdx.x)),
+          p1(SHARES ? a.first(blockIdx.x + 1, gridDim.x) : static_cast<int>(a.n_tasks)), s0(0), s1(0), begun(false) {}
+    __device__ __forceinline__ bool next(const TcArgs& a) {
+        if (p >= p1) return false;
+        if constexpr (!SHARES) {
+            tk = a.tasks ? a.tasks[p] : tc_task<NK>(p);
+            s1 = static_cast<int>((a.mols ? a.mols[tk.mol].nk_pad : a.single.nk_pad) / kTcKj);
+            p += gridDim.x;
+        } else {
+            const int np = a.pieces(), q = p / np, k = p - q * np, k1 = min(np, k + (p1 - p));
+            tk = tc_task<NK>(q);
+            p += k1 - k;
+            s0 = k * a.flush;
+            s1 = (k1 == np) ? a.n_stage() : k1 * a.flush;
+            begun = k > 0;
+        }
+        return true;
+    }
+};
 
 __device__ __forceinline__ void tmap_acquire(const CUtensorMap* m) {
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
@@ -192,7 +230,7 @@ __device__ __forceinline__ uint32_t a_col(int b) {
     return NK == 1 ? 384u + 64u * b : 256u + 128u * b;
 }
 
-template <int PQ, int NK>  // PQ accumulator columns per generator thread (= Ppad / 4)
+template <int PQ, int NK, bool SHARES>  // PQ accumulator columns per generator thread (= Ppad / 4)
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUtensorMap tm_ul,
           const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CUtensorMap tm_yl,
@@ -214,8 +252,6 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kTcRing + 6);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // a task = 128 rows of one molecule x (both kinds if NK == 2, else one kind)
-    const int64_t n_tiles = args.n_tasks;
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < kTcRing; ++b) {
@@ -245,8 +281,8 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
             bool ok = true;
             int cur_mol = -1;
             const CUtensorMap* mp[4] = {&tm_uh, &tm_ul, &tm_yh, &tm_yl};
-            for (int64_t q = blockIdx.x; q < n_tiles && ok; q += gridDim.x) {
-                const TcTask tk = tc_task<NK>(args, q);
+            for (TcWalk<NK, SHARES> w(args); ok && w.next(args);) {
+                const TcTask& tk = w.tk;
                 const TcMol M = args.mols ? args.mols[tk.mol] : args.single;
                 if (tk.mol != cur_mol) {  // a new molecule's tensor maps
                     cur_mol = tk.mol;
@@ -258,8 +294,7 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
                         tc::prefetch_tmap(mp[k]);
                     }
                 }
-                const int n_stage = static_cast<int>(M.nk_pad / kTcKj);
-                for (int s = 0; s < n_stage; ++s) {
+                for (int s = w.s0; s < w.s1; ++s) {
                     if (!wait_or_abort(&b_empty[slot], ph ^ 1u, args.err, abort_flag)) {
                         ok = false;
                         break;
@@ -291,12 +326,9 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
             int slot = 0, ab = 0;
             uint32_t ph = 0, aph = 0;
             bool ok = true, issued_any = false;
-            for (int64_t q = blockIdx.x; q < n_tiles && ok; q += gridDim.x) {
-                const TcTask tk = tc_task<NK>(args, q);
-                const int kind0 = tk.kind;
-                const int64_t nkp = args.mols ? args.mols[tk.mol].nk_pad : args.single.nk_pad;
-                const int n_stage = static_cast<int>(nkp / kTcKj);
-                for (int s = 0; s < n_stage; ++s) {
+            for (TcWalk<NK, SHARES> w(args); ok && w.next(args);) {
+                const int kind0 = w.tk.kind;
+                for (int s = w.s0; s < w.s1; ++s) {
                     if (!wait_or_abort(&a_full[ab], aph, args.err, abort_flag) ||
                         !wait_or_abort(&b_full[slot], ph, args.err, abort_flag)) {
                         ok = false;
@@ -395,7 +427,7 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
             return true;
         };
         // descriptor fields are read where they are used (not held across the stage loop)
-        auto flush = [&](int mol, int kind0, int64_t i) {
+        auto flush = [&](int mol, int kind0, int64_t i, bool begun, bool fresh) {
             const TcMol* mp = args.mols ? args.mols + mol : nullptr;
             const int64_t nk = mp ? mp->nk : args.single.nk;
             const int64_t nk_pad = mp ? mp->nk_pad : args.single.nk_pad;
@@ -410,11 +442,12 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
                 for (int c = 0; c < PQ; ++c) {
                     const int t = part * PQ + c;
                     if (i < nk && t < Pn) {
-                        double* o = acc_base + ((static_cast<int64_t>(kind) * acc_P + t0 + t) * nk_pad + i);
+                        double* o = begun ? args.side + ((static_cast<int64_t>(blockIdx.x) * NK + k) * PPAD + t) * 128 + quad * 32 + lane
+                                          : acc_base + ((static_cast<int64_t>(kind) * acc_P + t0 + t) * nk_pad + i);
                         const double v = static_cast<double>(acc[k][c]);
                         // the gamma accumulator holds -(T3 u + T4 y); streaming loads and
                         // stores keep the partial output from evicting the trial tiles
-                        __stcs(o, __ldcs(o) + ((kind == 0) ? v : -v));
+                        __stcs(o, (fresh ? 0.0 : __ldcs(o)) + ((kind == 0) ? v : -v));
                     }
                     acc[k][c] = 0.0f;
                 }
@@ -426,10 +459,9 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
         int pslot = 0;         // ring slot of the previous stage
         int dbuf = 0;          // accumulator buffer of the previous stage
         uint32_t dph = 0;      // and its phase bit
-        for (int64_t q = blockIdx.x; q < n_tiles && ok; q += gridDim.x) {
-            const TcTask tk = tc_task<NK>(args, q);
+        for (TcWalk<NK, SHARES> w(args); ok && w.next(args);) {
+            const TcTask& tk = w.tk;
             const TcMol* mp = args.mols ? args.mols + tk.mol : nullptr;
-            const int n_stage = static_cast<int>((mp ? mp->nk_pad : args.single.nk_pad) / kTcKj);
             const int kind0 = tk.kind;
             const int64_t i = static_cast<int64_t>(tk.row_tile) * 128 + quad * 32 + lane;
             float xi = 0.f, yi = 0.f, zi = 0.f, oi = 1.f, ki = 1.f, pi_ = 0.f, qi = 0.f;
@@ -442,7 +474,8 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
                           make_float2(oi, oi), make_float2(ki, ki), make_float2(-pi_, -pi_),
                           make_float2(-qi, -qi)};
             int until_flush = args.flush;
-            for (int s = 0; s < n_stage; ++s) {
+            bool fresh = w.begun;  // the side output holds nothing yet
+            for (int s = w.s0; s < w.s1; ++s) {
                 // operand buffer ab is free once the MMAs of the stage two back are done
                 bool got = wait_or_abort(&b_full[slot], ph, args.err, abort_flag);
                 got = got && wait_or_abort(&mma_done[ab], aph ^ 1u, args.err, abort_flag);
@@ -486,7 +519,7 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&a_full[ab]);  // hand the operands to the MMA issuer
                 // drain the previous stage while this stage's MMAs run
-                if (s > 0) {
+                if (s > w.s0) {
                     if (!drain(dbuf, dph, kind0)) {
                         ok = false;
                         break;
@@ -495,7 +528,8 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
                     // slot of the previous stage can be refilled
                     if (lane == 0) mbar_arrive(&b_empty[pslot]);
                     if (--until_flush == 0) {
-                        flush(tk.mol, kind0, i);
+                        flush(tk.mol, kind0, i, w.begun, fresh);
+                        fresh = false;
                         until_flush = args.flush;
                     }
                 }
@@ -515,7 +549,7 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
                 break;
             }
             if (lane == 0) mbar_arrive(&b_empty[pslot]);
-            flush(tk.mol, kind0, i);
+            flush(tk.mol, kind0, i, w.begun, fresh);
         }
         tc::wait_st();  // nothing of ours is in flight to TMEM on any exit path
         tc::wait_ld();
@@ -526,6 +560,28 @@ k_hess_tc(const __grid_constant__ CUtensorMap tm_uh, const __grid_constant__ CUt
     if (warp == kTcMmaWarp) {
         tc::fence_after();
         tc::tmem_dealloc(tmem, kTmemCols);
+    }
+}
+
+// Adds the side outputs of the CTAs whose shares began inside a task to its outputs, in CTA order.
+// Block = (task, trial), thread = row.
+template <int NK>
+__global__ void __launch_bounds__(128) k_hess_tc_join(TcArgs a, int ppad, int grid) {
+    const TcTask tk = tc_task<NK>(static_cast<int>(blockIdx.x));
+    const int t = static_cast<int>(blockIdx.y), np = a.pieces();
+    const int64_t i = static_cast<int64_t>(tk.row_tile) * 128 + threadIdx.x, b = static_cast<int64_t>(blockIdx.x) * np;
+    if (i >= a.single.nk) return;
+    double v[NK] = {};
+    // shares with b < first(c) < b + np (first(c) = floor(c all / grid))
+    for (int64_t c = (b * grid) / (a.n_tasks * np); c < grid; ++c) {
+        const int64_t f = a.first(c, grid);
+        if (f <= b) continue;
+        if (f >= b + np) break;
+        for (int k = 0; k < NK; ++k) v[k] += a.side[((c * NK + k) * ppad + t) * 128 + threadIdx.x];
+    }
+    for (int k = 0; k < NK; ++k) {
+        const int kind = NK == 2 ? k : tk.kind;
+        a.single.acc[(static_cast<int64_t>(kind) * a.single.acc_P + a.single.t0 + t) * a.single.nk_pad + i] += v[k];
     }
 }
 
@@ -598,38 +654,61 @@ int hess_tc_ppad(int32_t P) {
     return p < 32 ? 32 : p;
 }
 
-template <int PQ, int NK>
+template <int PQ, int NK, bool SHARES>
 static cudaError_t launch_tc_t(const CUtensorMap* maps, const TcArgs& a, int n_sm, cudaStream_t st) {
     const TcSmemLayout L = tc_layout(4 * PQ);
-    cudaError_t e = cudaFuncSetAttribute(k_hess_tc<PQ, NK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_hess_tc<PQ, NK, SHARES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L.total));
     if (e != cudaSuccess) return e;
-    const int grid = static_cast<int>(a.n_tasks < n_sm ? a.n_tasks : n_sm);
+    const int64_t all = a.n_tasks * (SHARES ? a.pieces() : 1);
+    const int grid = static_cast<int>(all < n_sm ? all : n_sm);
     if (grid <= 0) return cudaSuccess;
-    k_hess_tc<PQ, NK><<<grid, kTcThreads, L.total, st>>>(maps[0], maps[1], maps[2], maps[3], a);
+    k_hess_tc<PQ, NK, SHARES><<<grid, kTcThreads, L.total, st>>>(maps[0], maps[1], maps[2], maps[3], a);
+    if ((e = cudaGetLastError()) != cudaSuccess || !SHARES) return e;
+    k_hess_tc_join<NK><<<dim3(static_cast<unsigned>(a.n_tasks), static_cast<unsigned>(a.single.Pn)), 128, 0, st>>>(
+        a, 4 * PQ, grid);
     return cudaGetLastError();
 }
 
 // Both kinds share a tile whenever both accumulators fit in TMEM (Ppad <= 64).
 int hess_tc_kinds_per_tile(int ppad) { return ppad <= 64 ? 2 : 1; }
 
-static cudaError_t launch_tc_dispatch(int ppad, const CUtensorMap* maps, const TcArgs& a, int n_sm,
+template <bool SHARES>
+static cudaError_t launch_tc_width(int ppad, const CUtensorMap* maps, const TcArgs& a, int n_sm,
                                       cudaStream_t st) {
     switch (ppad / 4) {
-        case 8: return launch_tc_t<8, 2>(maps, a, n_sm, st);
-        case 16: return launch_tc_t<16, 2>(maps, a, n_sm, st);
-        case 24: return launch_tc_t<24, 1>(maps, a, n_sm, st);
-        case 32: return launch_tc_t<32, 1>(maps, a, n_sm, st);
-        case 40: return launch_tc_t<40, 1>(maps, a, n_sm, st);
-        case 48: return launch_tc_t<48, 1>(maps, a, n_sm, st);
+        case 8: return launch_tc_t<8, 2, SHARES>(maps, a, n_sm, st);
+        case 16: return launch_tc_t<16, 2, SHARES>(maps, a, n_sm, st);
+        case 24: return launch_tc_t<24, 1, SHARES>(maps, a, n_sm, st);
+        case 32: return launch_tc_t<32, 1, SHARES>(maps, a, n_sm, st);
+        case 40: return launch_tc_t<40, 1, SHARES>(maps, a, n_sm, st);
+        case 48: return launch_tc_t<48, 1, SHARES>(maps, a, n_sm, st);
         default: return cudaErrorInvalidValue;
     }
+}
+
+static cudaError_t launch_tc_dispatch(int ppad, const CUtensorMap* maps, const TcArgs& a, int n_sm, cudaStream_t st) {
+    return a.side ? launch_tc_width<true>(ppad, maps, a, n_sm, st) : launch_tc_width<false>(ppad, maps, a, n_sm, st);
+}
+
+static int64_t tc_tasks(int64_t nk, int ppad) {
+    return (hess_tc_kinds_per_tile(ppad) == 2 ? 1 : 2) * ((nk + 127) / 128);
+}
+
+// Doubles of `side` for equal shares of a launch of Pn trials; 0 where whole tasks are dealt.  Equal shares
+// take 0 to 4 % longer per stage (registers) and a join: milliseconds of the call, whole tasks and shares,
+// 41,000 points P = 54 9.33, 7.12, P = 180 14.46, 14.14; 29,778 points 4.58, 4.27 and 8.48, 7.79; 38,912 points
+// (whole rounds: not taken) 5.96, 5.99 and 11.09, 11.43.
+size_t hess_tc_side(int64_t nk, int64_t nk_pad, int32_t Pn, int flush, int n_sm) {
+    const int ppad = hess_tc_ppad(Pn);
+    if (!shares_pay(tc_tasks(nk, ppad), nk_pad / kTcKj, flush > 0 ? flush : 512, n_sm)) return 0;
+    return static_cast<size_t>(n_sm) * hess_tc_kinds_per_tile(ppad) * static_cast<size_t>(ppad) * 128;
 }
 
 // Contract the trials [t0, t0 + Pn) (Pn <= 192) of one system; split arrays have `rows` rows.
 cudaError_t launch_hess_tc(const PointsDev& p, int32_t Pn, int32_t t0, int64_t acc_P,
                            const float* uh, const float* ul, const float* yh, const float* yl,
-                           int64_t rows, int n_sm, int flush, double* acc, int* err,
+                           int64_t rows, int n_sm, int flush, double* acc, double* side, int* err,
                            cudaStream_t st) {
     if (p.nk == 0) return cudaSuccess;
     const int ppad = hess_tc_ppad(Pn);
@@ -642,8 +721,9 @@ cudaError_t launch_hess_tc(const PointsDev& p, int32_t Pn, int32_t t0, int64_t a
     a.single = TcMol{p.r32a, p.r32b, p.r32p, nullptr, acc, p.nk, p.nk_pad, acc_P, Pn, t0};
     a.mols = nullptr;
     a.tasks = nullptr;
-    a.n_tasks = (hess_tc_kinds_per_tile(ppad) == 2 ? 1 : 2) * ((p.nk + 127) / 128);
+    a.n_tasks = tc_tasks(p.nk, ppad);
     a.flush = flush > 0 ? flush : 512;
+    a.side = side;
     a.err = err;
     return launch_tc_dispatch(ppad, maps, a, n_sm, st);
 }
@@ -671,6 +751,7 @@ cudaError_t launch_hess_tc_batch(const void* mols, const void* tasks, int64_t n_
     a.tasks = static_cast<const TcTask*>(tasks);
     a.n_tasks = n_tasks;
     a.flush = flush > 0 ? flush : 512;
+    a.side = nullptr;
     a.err = err;
     return launch_tc_dispatch(ppad, unused, a, n_sm, st);
 }

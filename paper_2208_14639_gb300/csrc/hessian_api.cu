@@ -1,5 +1,7 @@
 // Orchestration of vv10_hessian_contract (Sec. II.B, Eq. frhot): A/B/C row sums for the
 // delta_ij/w_i terms, trial preparation, the pair-part contraction and the epilogue.
+#include <algorithm>
+
 #include "kernels.hpp"
 #include "vv10_internal.hpp"
 
@@ -148,16 +150,27 @@ vv10_status vv10_ctx::tc_contract(int32_t Pn, int cap, cudaStream_t st) {
                "trial split");
     }
     const size_t ab = sizeof(double) * 2 * static_cast<size_t>(Pn) * P.nk_pad;
-    H_TRY(ensure(hacc, ab, "contraction partials"));
+    // equal shares of the stages need a side output after the partials; without room (or in a
+    // capture, where nothing can be allocated), whole tasks
+    auto group = [&](int g) { return std::min(pg, Pn - g * pg); };
+    auto side_n = [&](int g) { return hess_tc_side(P.nk, P.nk_pad, group(g), tc_flush, n_sm); };
+    const size_t sd = sizeof(double) * std::max(side_n(0), side_n(ng - 1));
+    const bool shares = sd > 0 && (hacc.bytes >= ab + sd || !stream_capturing(st)) &&
+                        ensure(hacc, ab + sd, "contraction partials") == VV10_OK;
+    if (!shares) H_TRY(ensure(hacc, ab, "contraction partials"));
+    set_error("");
+    double* side = shares ? reinterpret_cast<double*>(static_cast<char*>(hacc.p) + ab) : nullptr;
     H_CUDA(cudaMemsetAsync(hacc.p, 0, ab, st), "zero contraction partials");
-    PhaseScope ph(this, PH_CONTRACT_TC, st, ng);
+    int launches = ng;
+    for (int g = 0; g < ng; ++g) launches += side && side_n(g) > 0;
+    PhaseScope ph(this, PH_CONTRACT_TC, st, launches);
     for (int g = 0; g < ng; ++g) {
-        const int t0 = g * pg;
-        const int pn = (Pn - t0 < pg) ? Pn - t0 : pg;
+        const int t0 = g * pg, pn = group(g);
         H_CUDA(launch_hess_tc(P, pn, t0, Pn, static_cast<float*>(tc_uh.p),
                               static_cast<float*>(tc_ul.p), static_cast<float*>(tc_yh.p),
                               static_cast<float*>(tc_yl.p), rows, n_sm, tc_flush,
-                              static_cast<double*>(hacc.p), static_cast<int*>(dev_err.p), st),
+                              static_cast<double*>(hacc.p), side_n(g) > 0 ? side : nullptr,
+                              static_cast<int*>(dev_err.p), st),
                "tensor-core contraction");
     }
     return VV10_OK;

@@ -240,9 +240,25 @@ cudaError_t launch_trial_tc_batch(const EpiMol* mols, const int64_t* pre, int n_
 // partial output acc [2][acc_P][nk_pad] (zeroed by the caller).  uh/ul/yh/yl: FP32
 // [rows][nk_pad] hi/lo parts of u and y; `flush` = stages between FP64 flushes.
 int hess_tc_ppad(int32_t P);
+// Whether equal shares of the pieces of `flush` stages beat whole tasks dealt in turn: the longest share is
+// at least 5 % shorter than the whole tasks of the longest CTA.
+inline bool shares_pay(int64_t n_tasks, int64_t n_stage, int64_t flush, int64_t n_sm) {
+    const int64_t np = (n_stage + flush - 1) / flush, all = n_tasks * np;
+    if (np <= 1 || n_sm <= 0) return false;
+    const int64_t grid = all < n_sm ? all : n_sm, whole = (n_tasks + n_sm - 1) / n_sm * n_stage;
+    int64_t worst = 0;
+    for (int64_t c = 0; c < grid; ++c) {
+        const int64_t p0 = c * all / grid, p1 = (c + 1) * all / grid;
+        const int64_t w = (p1 - p0) * flush - (p1 / np - p0 / np) * (np * flush - n_stage);
+        worst = w > worst ? w : worst;
+    }
+    return 20 * worst <= 19 * whole;
+}
+// `side`: hess_tc_side doubles, or null (whole tasks are dealt to the CTAs).
+size_t hess_tc_side(int64_t nk, int64_t nk_pad, int32_t Pn, int flush, int n_sm);
 cudaError_t launch_hess_tc(const PointsDev& p, int32_t Pn, int32_t t0, int64_t acc_P,
                            const float* uh, const float* ul, const float* yh, const float* yl,
-                           int64_t rows, int n_sm, int flush, double* acc, int* err,
+                           int64_t rows, int n_sm, int flush, double* acc, double* side, int* err,
                            cudaStream_t st);
 
 // Tensor-core split-FP16 contraction (hess_f16.cu).  chunk_bytes: trial-tile bytes of one j
