@@ -3,7 +3,10 @@
 // quantity and one tensor-core launch per trial-count class, and replayable as a CUDA graph.
 #include <algorithm>
 #include <cstring>
+#include <functional>
 #include <numeric>
+#include <queue>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -404,16 +407,27 @@ vv10_status vv10_ctx::batch_hess(vv10_precision prec, const int32_t* Pt, const d
                                  at<double>(B.acc, M.acc), M.nk, M.nk_pad, M.n_t, pn, t0);
             }
             const int kinds = hess_tc_kinds_per_tile(ppad) == 2 ? 1 : 2;
-            std::vector<unsigned char> tk;
             int64_t nt = 0;
+            for (const auto& g : groups) nt += kinds * ((B.mol[g.first].nk + 127) / 128);
+            std::vector<unsigned char> tk(hess_tc_task_bytes() * static_cast<size_t>(nt));
+            // CTA b runs the table's tasks b, b + G, ...: each task, longest first, goes to the CTA with the
+            // least work so far that has a slot left.  (In the order of the molecules CTA 0 had the longest
+            // task of every round.)
+            const int64_t G = std::min<int64_t>(nt, n_sm);
+            using Load = std::pair<int64_t, int64_t>;  // stages dealt, CTA
+            std::priority_queue<Load, std::vector<Load>, std::greater<Load>> least;
+            std::vector<int64_t> used(static_cast<size_t>(G), 0);
+            for (int64_t b = 0; b < G; ++b) least.push({0, b});
             for (size_t k = 0; k < groups.size(); ++k) {
-                const int64_t rt = (B.mol[groups[k].first].nk + 127) / 128;
-                for (int64_t r = 0; r < rt; ++r)
+                const BatchMol& M = B.mol[groups[k].first];
+                for (int64_t r = 0; r < (M.nk + 127) / 128; ++r)
                     for (int kind = 0; kind < kinds; ++kind) {
-                        tk.resize(tk.size() + hess_tc_task_bytes());
-                        hess_tc_fill_task(tk.data() + hess_tc_task_bytes() * nt, static_cast<int32_t>(k),
+                        const Load l = least.top();
+                        least.pop();
+                        const int64_t q = l.second + G * used[l.second]++;
+                        hess_tc_fill_task(tk.data() + hess_tc_task_bytes() * q, static_cast<int32_t>(k),
                                           static_cast<int32_t>(r), kind);
-                        ++nt;
+                        if (l.second + G * used[l.second] < nt) least.push({l.first + M.nk_pad, l.second});
                     }
             }
             c.tasks = a256(tab.size());
