@@ -61,10 +61,10 @@ typedef enum {
                                (per trial column; per row and 32-j stage for the kernel
                                tiles); elsewhere as VV10_MIXED_TF32X3                       */
     VV10_FP64_TC = 4        /* as VV10_FP64, except the pair part of the Hessian contraction:
-                               kernel tiles generated in FP64 and the trials are cut into five
-                               8-bit integer slices each (FP16-exact), whose 15 leading
-                               products the tensor cores sum exactly in FP32 (about 40 bits
-                               of each tile and trial kept); results agree with VV10_FP64 to
+                               kernel tiles generated in double-FP32 and the trials are cut
+                               into seven 8-bit integer slices each (FP16-exact), whose 28
+                               leading products the tensor cores sum exactly in FP32, up to
+                               64 trials a launch; results agree with VV10_FP64 to
                                ~1e-11 relative in norm, each element to ~1e-10 of its size
                                (the double-FP32 tiles carry ~46 bits).  Single systems only:
                                the batched contraction returns VV10_ERR_UNSUPPORTED.       */
