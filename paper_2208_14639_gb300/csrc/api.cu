@@ -898,9 +898,11 @@ vv10_status vv10_weight_response(vv10_handle h, vv10_precision prec, int32_t P,
         const int32_t rows = ng * ppad;
         const size_t nsplit = static_cast<size_t>(rows) * static_cast<size_t>(Pd.nk_pad);
         // nsplit is a multiple of 32 x 64: the side outputs after the split stay aligned
-        const size_t side_n = weight_tc_side(Pd.nk_pad, ppad, h->n_sm);
-        bool shares = side_n > 0 && h->ensure(h->wsplit, 2 * sizeof(float) * nsplit + sizeof(double) * side_n,
-                                              "weight direction split") == VV10_OK;
+        const size_t side_n = weight_tc_side(Pd.nk, Pd.nk_pad, ng, ppad, h->n_sm);
+        const size_t with_side = 2 * sizeof(float) * nsplit + sizeof(double) * side_n;
+        // without room (or in a capture, where nothing can be allocated) whole tasks are dealt
+        const bool shares = side_n > 0 && (h->wsplit.bytes >= with_side || !stream_capturing(st)) &&
+                            h->ensure(h->wsplit, with_side, "weight direction split") == VV10_OK;
         if (!shares) VV10_TRY(h->ensure(h->wsplit, 2 * sizeof(float) * nsplit, "weight direction split"));
         h->set_error("");
         float* yh = static_cast<float*>(h->wsplit.p);

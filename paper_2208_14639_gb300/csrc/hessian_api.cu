@@ -244,7 +244,8 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
                "FP64 trial slices");
     }
     const size_t ab = sizeof(double) * 2 * static_cast<size_t>(Pn) * P.nk_pad;
-    H_TRY(ensure(hacc, ab + sizeof(double) * 128 * static_cast<size_t>(pg) * n_sm, "contraction partials"));
+    // side outputs for the widest launch, whatever pg: the buffer never has to grow for fewer trials
+    H_TRY(ensure(hacc, ab + sizeof(double) * 128 * static_cast<size_t>(cap) * n_sm, "contraction partials"));
     H_CUDA(cudaMemsetAsync(hacc.p, 0, ab, st), "zero contraction partials");
     const int64_t civ_group = civ_n / ng;
     PhaseScope ph(this, PH_CONTRACT_TC, st, ng);

@@ -387,10 +387,10 @@ cudaError_t launch_weight_response(const PointsDev& p, bool fp64, int32_t Pn, co
 void weight_tc_groups(int32_t P, int* n_groups, int* ppad);
 cudaError_t launch_weight_split(const double* yk, int32_t Pn, int32_t rows, int64_t nk_pad,
                                 float* yh, float* yl, cudaStream_t st);
+// `side`: weight_tc_side doubles, or null (whole tasks are dealt to the CTAs).
+size_t weight_tc_side(int64_t nk, int64_t nk_pad, int n_groups, int ppad, int n_sm);
 cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, const float* yl,
                              int32_t rows, double* E, double* U, double* W, int n_sm, double* side, int* err,
-// `side`: weight_tc_side doubles, or null (whole tasks are dealt to the CTAs).
-size_t weight_tc_side(int64_t nk_pad, int ppad, int n_sm);
                              cudaStream_t st);
 // 2-D tensor map over a [rows][nk_pad] FP32 array, box 16 j x ppad rows, 64-byte swizzle.
 bool tc_make_map_f32(void* out /* CUtensorMap */, const float* base, int64_t nk_pad, int64_t rows,

@@ -85,16 +85,18 @@ struct WtArgs {
     double* side;         // [CTA][kind][Ppad][128] output of a share's first task if it is a begun one
     int* err;
     // Shares: the pieces of `flush` stages (what one FP64 flush sums) in the order (task, piece) are
-    // dealt evenly; without `side` a piece is a whole task.
+    // dealt evenly.
     __host__ __device__ int n_stage() const { return static_cast<int>(nk_pad / kWtKj); }
-    __host__ __device__ int pieces() const { return side ? (n_stage() + flush - 1) / flush : 1; }  // of a task
-    __host__ __device__ int64_t first(int64_t cta, int64_t grid) const { return cta * (n_tasks * pieces()) / grid; }
+    __host__ __device__ int pieces() const { return (n_stage() + flush - 1) / flush; }  // of a task
+    __host__ __device__ int first(int64_t cta, int64_t grid) const {
+        return static_cast<int>(cta * (n_tasks * pieces()) / grid);
+    }
 };
 
-// The segments of a CTA's share: task q, stages s0 .. s1 - 1 (begun: not the task's first ones).
+// With SHARES a CTA's segments: task q, stages s0 .. s1 - 1 (begun: not the task's first ones).  (Whole tasks
+// keep a plain loop: through this walk they took 1.5 % longer at 64 directions.)
 struct WtWalk {
-    int64_t p, p1, q;
-    int s0, s1;
+    int p, p1, q, s0, s1;
     bool begun;
     __device__ __forceinline__ explicit WtWalk(const WtArgs& a)
         : p(a.first(blockIdx.x, gridDim.x)), p1(a.first(blockIdx.x + 1, gridDim.x)), q(0), s0(0), s1(0), begun(false) {}
@@ -102,8 +104,7 @@ struct WtWalk {
         if (p >= p1) return false;
         const int np = a.pieces();
         q = p / np;
-        const int k = static_cast<int>(p - q * np);
-        const int k1 = static_cast<int>(min(static_cast<int64_t>(np), k + (p1 - p)));
+        const int k = p - q * np, k1 = min(np, k + (p1 - p));
         p += k1 - k;
         s0 = k * a.flush;
         s1 = (k1 == np) ? a.n_stage() : k1 * a.flush;
@@ -161,7 +162,7 @@ __device__ __forceinline__ uint32_t tf32_hi_bits(float x) {
 // TMEM accumulator of kind k, buffer b.
 __device__ __forceinline__ uint32_t wt_dcol(int k, int b) { return 64u * (2 * k + b); }
 
-template <int PQ>  // accumulator columns per generator thread and kind (= Ppad / 4)
+template <int PQ, bool SHARES>  // accumulator columns per generator thread and kind (= Ppad / 4)
 __global__ void __launch_bounds__(kWtThreads, 1)
 k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CUtensorMap tm_yl,
            WtArgs args) {
@@ -181,6 +182,7 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kWtRing + 6);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n_stage = static_cast<int>(args.nk_pad / kWtKj);
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < kWtRing; ++b) {
@@ -210,9 +212,10 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             uint32_t ph = 0;
             int64_t issued = 0;
             bool ok = true;
-            for (WtWalk w(args); ok && w.next(args);) {
-                const int t0 = static_cast<int>(w.q % args.n_groups) * PPAD;
-                for (int s = w.s0; s < w.s1; ++s) {
+            WtWalk w(args);
+            for (int64_t q = blockIdx.x; (SHARES ? w.next(args) : q < args.n_tasks) && ok; q += gridDim.x) {
+                const int t0 = static_cast<int>((SHARES ? w.q : q) % args.n_groups) * PPAD;
+                for (int s = SHARES ? w.s0 : 0; s < (SHARES ? w.s1 : n_stage); ++s) {
                     if (!wt_wait(&b_empty[slot], ph ^ 1u, args.err, abort_flag)) {
                         ok = false;
                         break;
@@ -243,8 +246,9 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             int slot = 0, ab = 0;
             uint32_t ph = 0, aph = 0;
             bool ok = true, issued_any = false;
-            for (WtWalk w(args); ok && w.next(args);) {
-                for (int s = w.s0; s < w.s1; ++s) {
+            WtWalk w(args);
+            for (int64_t q = blockIdx.x; (SHARES ? w.next(args) : q < args.n_tasks) && ok; q += gridDim.x) {
+                for (int s = SHARES ? w.s0 : 0; s < (SHARES ? w.s1 : n_stage); ++s) {
                     if (!wt_wait(&a_full[ab], aph, args.err, abort_flag) ||
                         !wt_wait(&b_full[slot], ph, args.err, abort_flag)) {
                         ok = false;
@@ -334,9 +338,13 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
                     const int t = t0 + part * PQ + c;
                     if (o && row_ok && t < args.P) {
                         const double v = static_cast<double>(acc[k][c]);
-                        double* x = begun ? args.side + ((static_cast<int64_t>(blockIdx.x) * kWtKinds + k) * PPAD + t - t0) * 128 + r
-                                          : o + static_cast<int64_t>(t) * args.n + oi;
-                        *x = (fresh ? 0.0 : *x) + ((k == 0) ? v : -v);
+                        if constexpr (SHARES) {
+                            double* x = begun ? args.side + ((static_cast<int64_t>(blockIdx.x) * kWtKinds + k) * PPAD + t - t0) * 128 + r
+                                              : o + static_cast<int64_t>(t) * args.n + oi;
+                            *x = (fresh ? 0.0 : *x) + ((k == 0) ? v : -v);
+                        } else {
+                            o[static_cast<int64_t>(t) * args.n + oi] += (k == 0) ? v : -v;
+                        }
                     }
                     acc[k][c] = 0.0f;
                 }
@@ -347,9 +355,10 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
         uint32_t ph = 0, aph = 0;
         int pslot = 0, dbuf = 0;
         uint32_t dph = 0;
-        for (WtWalk w(args); ok && w.next(args);) {
-            const int64_t row_tile = w.q / args.n_groups;
-            const int t0 = static_cast<int>(w.q % args.n_groups) * PPAD;
+        WtWalk w(args);
+        for (int64_t q = blockIdx.x; (SHARES ? w.next(args) : q < args.n_tasks) && ok; q += gridDim.x) {
+            const int64_t row_tile = (SHARES ? w.q : q) / args.n_groups;
+            const int t0 = static_cast<int>((SHARES ? w.q : q) % args.n_groups) * PPAD;
             const int64_t i = row_tile * 128 + r;
             float xi = 0.f, yi = 0.f, zi = 0.f, oi = 1.f, ki = 1.f;
             if (i < args.nk) {
@@ -360,8 +369,8 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             const float2 X = make_float2(xi, xi), Y = make_float2(yi, yi), Z = make_float2(zi, zi);
             const float2 O = make_float2(oi, oi), K = make_float2(ki, ki);
             int until_flush = args.flush;
-            bool fresh = w.begun;  // the side output holds nothing yet
-            for (int s = w.s0; s < w.s1; ++s) {
+            bool fresh = SHARES && w.begun;  // the side output holds nothing yet
+            for (int s = SHARES ? w.s0 : 0; s < (SHARES ? w.s1 : n_stage); ++s) {
                 // operand buffer ab is free once the MMAs of the stage two back are done
                 bool got = wt_wait(&b_full[slot], ph, args.err, abort_flag);
                 got = got && wt_wait(&mma_done[ab], aph ^ 1u, args.err, abort_flag);
@@ -399,14 +408,14 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&a_full[ab]);
                 // drain the previous stage while this stage's MMAs run
-                if (s > w.s0) {
+                if (s > (SHARES ? w.s0 : 0)) {
                     if (!drain(dbuf, dph)) {
                         ok = false;
                         break;
                     }
                     if (lane == 0) mbar_arrive(&b_empty[pslot]);
                     if (--until_flush == 0) {
-                        flush(t0, i, w.begun, fresh);
+                        flush(t0, i, SHARES && w.begun, SHARES && fresh);
                         fresh = false;
                         until_flush = args.flush;
                     }
@@ -427,7 +436,7 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
                 break;
             }
             if (lane == 0) mbar_arrive(&b_empty[pslot]);
-            flush(t0, i, w.begun, fresh);
+            flush(t0, i, SHARES && w.begun, SHARES && fresh);
         }
         tc::wait_st();  // nothing of ours is in flight to or from TMEM on any exit path
         tc::wait_ld();
@@ -478,17 +487,17 @@ __global__ void k_wdir_split(const double* __restrict__ yk, int32_t Pn, int64_t 
     yl[o] = a - ah;
 }
 
-template <int PQ>
+template <int PQ, bool SHARES>
 cudaError_t launch_wt(const CUtensorMap* maps, const WtArgs& a, int n_sm, cudaStream_t st) {
     const WtLayout L = wt_layout(4 * PQ);
-    cudaError_t e = cudaFuncSetAttribute(k_wresp_tc<PQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_wresp_tc<PQ, SHARES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L.total));
     if (e != cudaSuccess) return e;
-    const int64_t all = a.n_tasks * a.pieces();
+    const int64_t all = a.n_tasks * (SHARES ? a.pieces() : 1);
     const int grid = static_cast<int>(all < n_sm ? all : n_sm);
     if (grid <= 0) return cudaSuccess;
-    k_wresp_tc<PQ><<<grid, kWtThreads, L.total, st>>>(maps[0], maps[1], a);
-    if ((e = cudaGetLastError()) != cudaSuccess || a.pieces() == 1) return e;
+    k_wresp_tc<PQ, SHARES><<<grid, kWtThreads, L.total, st>>>(maps[0], maps[1], a);
+    if ((e = cudaGetLastError()) != cudaSuccess || !SHARES) return e;
     k_wresp_join<<<dim3(static_cast<unsigned>(a.n_tasks), 4 * PQ), 128, 0, st>>>(a, 4 * PQ, grid);
     return cudaGetLastError();
 }
@@ -511,10 +520,12 @@ cudaError_t launch_weight_split(const double* yk, int32_t Pn, int32_t rows, int6
     return cudaGetLastError();
 }
 
-// Doubles of `side` for equal shares of the stages; 0 where a task is one piece, and whole tasks are dealt.
-// (Whole tasks at 39,542 kept points, 36 directions: 309 on 152 SMs, three rounds for 2.03.)
-size_t weight_tc_side(int64_t nk_pad, int ppad, int n_sm) {
-    return nk_pad > kWtFlush * kWtKj ? static_cast<size_t>(n_sm) * kWtKinds * static_cast<size_t>(ppad) * 128 : 0;
+// Doubles of `side` for equal shares of the stages; 0 where whole tasks are dealt.  Equal shares take about
+// 2 % longer per stage (registers) and a join: milliseconds of the call, whole tasks and shares, 41,000
+// points P = 18 7.21, 5.41, P = 54 7.80, 5.87; 38,912 points (two whole rounds) 4.57, 4.64 and 4.91, 5.02.
+size_t weight_tc_side(int64_t nk, int64_t nk_pad, int n_groups, int ppad, int n_sm) {
+    if (!shares_pay(static_cast<int64_t>(n_groups) * ((nk + 127) / 128), nk_pad / kWtKj, kWtFlush, n_sm)) return 0;
+    return static_cast<size_t>(n_sm) * kWtKinds * static_cast<size_t>(ppad) * 128;
 }
 
 cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, const float* yl,
@@ -545,7 +556,8 @@ cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, co
     a.flush = kWtFlush;
     a.side = side;
     a.err = err;
-    return ppad == 32 ? launch_wt<8>(maps, a, n_sm, st) : launch_wt<16>(maps, a, n_sm, st);
+    if (side) return ppad == 32 ? launch_wt<8, true>(maps, a, n_sm, st) : launch_wt<16, true>(maps, a, n_sm, st);
+    return ppad == 32 ? launch_wt<8, false>(maps, a, n_sm, st) : launch_wt<16, false>(maps, a, n_sm, st);
 }
 
 }  // namespace vv10
