@@ -57,9 +57,8 @@ FP32_LANES_PER_SM = 128
 ALU_OPS_PER_PAIR_TC = 40
 # the same when each output kind has its own tile generation (Ppad > 64): 2 x (25 + 5.5 + 2)
 ALU_OPS_PER_PAIR_TC_SPLIT = 65
-#   plain energy/potential pass: 13 shared (R^2, g, g', s, g g' s, reciprocal with its Newton
-#   step, Phi c) + 7 (1/s + 1/g and the three sums)
-ALU_OPS_PER_PAIR_EUW = 20
+#   energy/potential pass over unordered pairs: 29 operations serve both ordered pairs
+ALU_OPS_PER_PAIR_EUW = 14.5
 #   grid-grid Hessian block D_i^B: the same 13 shared, 10 for 1/(g g'), 1/s, omega_i/g,
 #   omega_j/g', (omega_i+omega_j)/s and D, 4 for the squared bracket, 4 for the scaled
 #   displacement, 6 outer-product and 1 identity-term accumulations
@@ -67,7 +66,7 @@ ALU_OPS_PER_PAIR_CH = 38
 #   weight-derivative sums: 19 to form 1/(g g' s), 1/s + 1/g and the three kernel values,
 #   then 3 FMAs per direction
 ALU_OPS_PER_PAIR_WR = 19
-#   FP64 tensor-core contraction, per pair, trial group of 32 and output kind: 33 for the
+#   FP64 tensor-core contraction, per pair, trial group of 64 and output kind: 33 for the
 #   exact coordinate differences and r^2, about 250 for the double-FP32 kernel tiles (17
 #   additions of 11 operations, 24 products of 7, a reciprocal of 12), 2 x 30 for the seven
 #   slices of the two tiles, and 8 x 40 / 4 for the level drains of the row's outputs
@@ -693,14 +692,14 @@ def gpu_arm(args):
     if dom == "contraction_tensor_core" and prec == vv.VV10_FP64_TC:
         # FP32 ALU-bound: double-FP32 tile generation, slicing and level drains
         t = per[dom] / 1e3
-        groups = -(-pb.P // 32)
+        groups = -(-pb.P // 64)
         alu_peak = N_SM * FP32_LANES_PER_SM * sm_mhz * 1e6
         ops = O64_ALU_OPS_PER_PAIR * groups * pairs_call
         roof = {"bound": "alu", "achieved": ops / t / 1e12, "peak": alu_peak / 1e12,
                 "unit": "Tops/s (FP32)", "frac": ops / t / alu_peak, "traffic": None,
                 "kernel": "k_hess_o64",
                 "peak_source": f"{N_SM} SMs x {FP32_LANES_PER_SM} FP32 lanes x {sm_mhz:.0f} MHz",
-                "counting": f"{O64_ALU_OPS_PER_PAIR} FP32 operations per pair and trial group of 32 "
+                "counting": f"{O64_ALU_OPS_PER_PAIR} FP32 operations per pair and trial group of 64 "
                             "(both output kinds)"}
     elif dom == "contraction_tensor_core":
         t = per[dom] / 1e3
