@@ -182,7 +182,12 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kWtRing + 6);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_stage = static_cast<int>(args.nk_pad / kWtKj);
+    const int n_stage = SHARES ? 0 : static_cast<int>(args.nk_pad / kWtKj);
+    // the task of a loop below, in its own width (a 64-bit division costs the shares registers)
+    auto task = [](const WtWalk& w, int64_t q) {
+        if constexpr (SHARES) return w.q;
+        else return q;
+    };
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < kWtRing; ++b) {
@@ -213,8 +218,8 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             int64_t issued = 0;
             bool ok = true;
             WtWalk w(args);
-            for (int64_t q = blockIdx.x; (SHARES ? w.next(args) : q < args.n_tasks) && ok; q += gridDim.x) {
-                const int t0 = static_cast<int>((SHARES ? w.q : q) % args.n_groups) * PPAD;
+            for (int64_t q = blockIdx.x; SHARES ? ok && w.next(args) : q < args.n_tasks && ok; q += gridDim.x) {
+                const int t0 = static_cast<int>(task(w, q) % args.n_groups) * PPAD;
                 for (int s = SHARES ? w.s0 : 0; s < (SHARES ? w.s1 : n_stage); ++s) {
                     if (!wt_wait(&b_empty[slot], ph ^ 1u, args.err, abort_flag)) {
                         ok = false;
@@ -247,7 +252,7 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
             uint32_t ph = 0, aph = 0;
             bool ok = true, issued_any = false;
             WtWalk w(args);
-            for (int64_t q = blockIdx.x; (SHARES ? w.next(args) : q < args.n_tasks) && ok; q += gridDim.x) {
+            for (int64_t q = blockIdx.x; SHARES ? ok && w.next(args) : q < args.n_tasks && ok; q += gridDim.x) {
                 for (int s = SHARES ? w.s0 : 0; s < (SHARES ? w.s1 : n_stage); ++s) {
                     if (!wt_wait(&a_full[ab], aph, args.err, abort_flag) ||
                         !wt_wait(&b_full[slot], ph, args.err, abort_flag)) {
@@ -356,9 +361,9 @@ k_wresp_tc(const __grid_constant__ CUtensorMap tm_yh, const __grid_constant__ CU
         int pslot = 0, dbuf = 0;
         uint32_t dph = 0;
         WtWalk w(args);
-        for (int64_t q = blockIdx.x; (SHARES ? w.next(args) : q < args.n_tasks) && ok; q += gridDim.x) {
-            const int64_t row_tile = (SHARES ? w.q : q) / args.n_groups;
-            const int t0 = static_cast<int>((SHARES ? w.q : q) % args.n_groups) * PPAD;
+        for (int64_t q = blockIdx.x; SHARES ? ok && w.next(args) : q < args.n_tasks && ok; q += gridDim.x) {
+            const int64_t row_tile = task(w, q) / args.n_groups;
+            const int t0 = static_cast<int>(task(w, q) % args.n_groups) * PPAD;
             const int64_t i = row_tile * 128 + r;
             float xi = 0.f, yi = 0.f, zi = 0.f, oi = 1.f, ki = 1.f;
             if (i < args.nk) {
