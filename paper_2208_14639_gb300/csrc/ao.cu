@@ -188,17 +188,24 @@ int64_t ao_channels_per_chunk(int64_t nk, int32_t nbf, int32_t n_ch, size_t max_
 
 namespace {
 
-// One product C = A B^T (A M x K, B N x K, k slowest): on the tensor cores unless it is short.
+// C = A B^T (A M x K, B N x K, k slowest) by FP64 FMA, the splits limited by the split-K scratch
+// (work_elems doubles).
+cudaError_t fma_product(const AoGemm& g, int M, int N, int64_t K, const double* A, const double* B,
+                        double* C, cudaStream_t st) {
+    int s = gemm_abt_splits(M, N, K, g.n_sm);
+    const size_t per = static_cast<size_t>(M) * static_cast<size_t>(N);
+    const int cap = static_cast<int>(g.work_elems / (per > 0 ? per : 1));
+    s = s < cap ? s : (cap > 0 ? cap : 1);
+    return launch_gemm_abt(M, N, K, A, M, B, N, C, M, g.work, s, st);
+}
+
+// The same on the tensor cores unless it is short.
 cudaError_t ao_product(const AoGemm& g, int M, int N, int64_t K, const double* A, const double* B,
                        double* C, cudaStream_t st) {
     if (gemm_slices_applies(K))
         return launch_gemm_slices(M, N, K, A, M, B, N, C, M, g.work,
                                   gemm_slices_splits(M, N, K, g.n_sm, g.work_elems), g.expo, g.err, st);
-    int s = gemm_abt_splits(M, N, K, g.n_sm);  // limited by the split-K scratch (work_elems doubles)
-    const size_t per = static_cast<size_t>(M) * static_cast<size_t>(N);
-    const int cap = static_cast<int>(g.work_elems / (per > 0 ? per : 1));
-    s = s < cap ? s : (cap > 0 ? cap : 1);
-    return launch_gemm_abt(M, N, K, A, M, B, N, C, M, g.work, s, st);
+    return fma_product(g, M, N, K, A, B, C, st);
 }
 
 // The channel chunks of M = Phi^T Z + Z^T Phi: make_coef(c0, nc, coef) launches the kernel that writes
@@ -275,7 +282,11 @@ cudaError_t launch_fock_derivative(const PointsDev& p, const AoGemm& g, const Fo
                                         256, 0, st>>>(p, in, a0, coef);
                         });
     if (e != cudaSuccess) return e;
-    // (2) the derivatives of the basis functions
+    // (2) the derivatives of the basis functions.  Their products run in FP64 FMA: the factors' columns
+    // alternate between d_c phi and b . grad d_c phi (alpha phi + ... and phi), of which only one carries
+    // the weight, and the slices of gemm_slices.cu have one scale for 128 of them, set by the larger
+    // (water with an s function of exponent 15,330, an atom's points in any order: elements off by up to
+    // 1e-10 of their sum of absolute terms instead of 1e-15).
     double* R = LR;
     double* L = LR + 2 * ne;
     double* Kall = K2;
@@ -287,12 +298,12 @@ cudaError_t launch_fock_derivative(const PointsDev& p, const AoGemm& g, const Fo
         k_fa_left<<<gx, 256, 0, st>>>(p, in, c, L);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = ao_product(g, nbf, nbf, 2 * p.nk, L, R, Kall, st);
+        e = fma_product(g, nbf, nbf, 2 * p.nk, L, R, Kall, st);
         if (e != cudaSuccess) return e;
         for (int32_t A = 0; A < p.n_atom; ++A) {
             const int64_t s0 = seg[A], na = seg[A + 1] - seg[A];
             if (na > 0) {
-                e = ao_product(g, nbf, nbf, 2 * na, L + 2 * s0 * nbf, R + 2 * s0 * nbf, KA, st);
+                e = fma_product(g, nbf, nbf, 2 * na, L + 2 * s0 * nbf, R + 2 * s0 * nbf, KA, st);
                 if (e != cudaSuccess) return e;
             }
             k_fa_basis<<<gn, 256, 0, st>>>(nbf, A, in.bf_atom, Kall, na > 0 ? KA : nullptr,

@@ -980,7 +980,7 @@ static vv10_status ao_assemble(vv10_handle h, int32_t nbf, const double* phi, co
     VV10_TRY(h->ensure(h->aoz, sizeof(double) * (nk * (nbf + 4) * chunk + 1), "assembly operand"));
     VV10_TRY(h->ensure(h->aom, sizeof(double) * static_cast<size_t>(nbf) * nbf * chunk, "assembly products"));
     const size_t gw = ao_gemm_work_elems(nbf, chunk, h->n_sm);
-    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), 2 * P.nk), "assembly product partials"));
+    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), P.nk), "assembly product partials"));
     const AoGemm g{static_cast<double*>(h->aogw.p), gw, reinterpret_cast<int32_t*>(static_cast<double*>(h->aogw.p) + gw),
                    h->n_sm, static_cast<int*>(h->dev_err.p)};
     PhaseScope ph(h, PH_AO_ASSEMBLY, st, P.nk > 0 ? 1 + 4 * static_cast<int>((n_ch + chunk - 1) / chunk) : 0);
@@ -1065,7 +1065,7 @@ vv10_status vv10_fock_derivative(vv10_handle h, int32_t nbf, const double* phi,
     VV10_TRY(h->ensure(h->aom, sizeof(double) * nn * chunk, "assembly products"));
     VV10_TRY(h->ensure(h->aofa, sizeof(double) * (4 * nk * nbf + 2 * nn), "basis-derivative factors"));
     const size_t gw = ao_gemm_work_elems(nbf, chunk, h->n_sm);
-    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), 2 * P.nk), "assembly product partials"));
+    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), P.nk), "assembly product partials"));
     const AoGemm g{static_cast<double*>(h->aogw.p), gw, reinterpret_cast<int32_t*>(static_cast<double*>(h->aogw.p) + gw),
                    h->n_sm, static_cast<int*>(h->dev_err.p)};
     std::vector<int64_t> seg(static_cast<size_t>(P.n_atom) + 1);

@@ -2,7 +2,8 @@
 // Fock-matrix equation, Sec. II.B G^t and F^A): A is M x K and B is N x K, both stored with
 // their K index slowest (column k of A at A + k lda, the M values of a column contiguous),
 // C is M x N column-major.  M and N are basis-function counts (tens to a few thousand), K the
-// number of kept grid points; from 512 of them the tensor-core kernel of gemm_slices.cu runs instead.
+// number of kept grid points; products of the basis values from 512 points on run on the tensor-core
+// kernel of gemm_slices.cu instead.
 //
 // 64 x 64 tiles of C, 256 threads with 4 x 4 results each, 16 k per shared-memory step (both
 // operand tiles loaded with unit stride in m or n), the K range split over gridDim.z CTAs so
