@@ -18,6 +18,11 @@
 // FMAs rounds at every k.  Against 80-bit and wider sums the assembled matrices are off by 1.5e-16 to
 // 9e-16 (1,500 to 40,000 points), those of the FMA chains by 3e-16 to 3.5e-15.
 //
+// A row's 128 elements of which one is not finite, or 2^512 and more (the scales of two rows could
+// overflow), have no digits: its exponent is stored as kGsPlain, its products are left out, and the
+// reduction forms them by FP64 FMA, so that NaN and infinities end up where an FP64 product puts them.
+// (At the other end block sums below 2^-978 are zero.)
+//
 // A CTA owns a 128 x 64 tile of C and a range of blocks.  Eight warps cut both operands' tiles of
 // 32 k (8 rows per warp and pass, loads of 64 contiguous bytes; the rows' E from a pass of its own)
 // into swizzled shared memory, double-buffered, while one thread issues the 72 MMAs of the 32 k
@@ -39,6 +44,8 @@ namespace {
 constexpr int kGsM = 128, kGsN = 64, kGsK = 32;  // tile of C, k per stage
 constexpr int kGsBlk = 4;                        // stages per block (one scale per row)
 constexpr int kGsSlices = 8;
+constexpr int kGsBig = 1023 + 511;               // largest biased exponent that is cut into digits
+constexpr int kGsPlain = -4096;                  // the row's block is left to the reduction
 constexpr int kGsWarps = 8;                      // worker warps; warp 8 issues the MMAs
 constexpr int kGsThreads = 12 * 32;              // (three warps a scheduler: 168 registers a thread)
 constexpr uint32_t kGsABytes = kGsM * 64, kGsBBytes = kGsN * 64;  // one slice: 64-byte rows
@@ -52,7 +59,8 @@ struct GsArgs {
     int32_t n_blk, per_split;    // blocks in all, and of one split
     const double *A, *B;
     int64_t lda, ldb;
-    const int32_t *ea, *eb;      // [block][row] biased exponent of the row's largest |element|
+    const int32_t *ea, *eb;      // [block][row] biased exponent of the row's largest |element|, or kGsPlain
+    const int32_t* plain;        // not 0: some row's block is kGsPlain
     double* part;                // [split][N][M]
     int* err;
 };
@@ -78,9 +86,9 @@ __device__ __forceinline__ void gs_cut(const double* __restrict__ X, int64_t ld,
                                        uint8_t* base, uint32_t slice_bytes) {
     const int lane = threadIdx.x & 31;
     const int r = row0 + (lane & 7), kq = lane >> 3;
-    const bool real = first + r < rows;
     double x[8];
-    const int e = real ? emax[first + r] : 0;
+    const int e = first + r < rows ? emax[first + r] : kGsPlain;
+    const bool real = e >= 0;  // others: zeros
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int64_t k = k0 + 8 * kq + q;
@@ -181,7 +189,7 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
                         const double x = fma(dl, 0x1p-32, dh);
                         // times 2^(E_a + E_b - 2 (1023 + 5) - 24)
                         int e = er + (n0 + half * 32 + c0 + u < args.N ? ec[c0 + u] : 0);
-                        e = e < 0 ? 0 : (e > 2047 ? 2047 : e);
+                        e = e < 0 ? 0 : e;  // (kGsPlain: 0; at most 2 kGsBig - 1057)
                         acc[c0 + u] = fma(x, __hiloint2double(e << 20, 0), acc[c0 + u]);
                     }
                 }
@@ -253,9 +261,9 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
     }
 }
 
-// emax[block][row] = biased exponent of the row's largest |element| in the block's 128 k.
+// emax[block][row] = biased exponent of the row's largest |element| in the block's 128 k, or kGsPlain.
 __global__ void __launch_bounds__(256) k_exp_max(const double* __restrict__ X, int64_t ld, int rows, int64_t K,
-                                                 int32_t* __restrict__ emax) {
+                                                 int32_t* __restrict__ emax, int32_t* __restrict__ plain) {
     __shared__ int sh[4][64];
     const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
     const int r = blockIdx.y * 64 + c;
@@ -267,25 +275,37 @@ __global__ void __launch_bounds__(256) k_exp_max(const double* __restrict__ X, i
             if (k0 + k < K) e = max(e, (__double2hiint(X[(k0 + k) * ld + r]) >> 20) & 0x7ff);
     sh[g][c] = e;
     __syncthreads();
-    if (g == 0 && r < rows)
-        emax[static_cast<int64_t>(blockIdx.x) * rows + r] = max(max(sh[0][c], sh[1][c]), max(sh[2][c], sh[3][c]));
+    if (g == 0 && r < rows) {
+        e = max(max(sh[0][c], sh[1][c]), max(sh[2][c], sh[3][c]));
+        if (e > kGsBig) {
+            e = kGsPlain;
+            *plain = 1;  // every writer the same value
+        }
+        emax[static_cast<int64_t>(blockIdx.x) * rows + r] = e;
+    }
 }
 
-// C[m + n ldc] = sum over the splits, in split order.
-__global__ void k_slices_reduce(int M, int N, int n_split, const double* __restrict__ part,
-                                double* __restrict__ C, int64_t ldc) {
+// C[m + n ldc] = sum over the splits, in split order, and of the blocks that have no digits.
+__global__ void k_slices_reduce(GsArgs a, int n_split, double* __restrict__ C, int64_t ldc) {
     const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int64_t mn = static_cast<int64_t>(M) * N;
+    const int64_t mn = static_cast<int64_t>(a.M) * a.N;
     if (e >= mn) return;
+    const int64_t n = e / a.M, m = e % a.M;
     double s = 0.0;
-    for (int z = 0; z < n_split; ++z) s += part[z * mn + e];
-    C[(e / M) * ldc + e % M] = s;
+    for (int z = 0; z < n_split; ++z) s += a.part[z * mn + e];
+    if (*a.plain)
+        for (int64_t b = 0; b < a.n_blk; ++b) {
+            if (a.ea[b * a.M + m] >= 0 && a.eb[b * a.N + n] >= 0) continue;
+            const int64_t k1 = min(a.K, (b + 1) * kGsBlk * kGsK);
+            for (int64_t k = b * kGsBlk * kGsK; k < k1; ++k) s = fma(a.A[k * a.lda + m], a.B[k * a.ldb + n], s);
+        }
+    C[n * ldc + m] = s;
 }
 
 }  // namespace
 
-size_t gemm_slices_expo_ints(int64_t rows, int64_t K) {
-    return static_cast<size_t>(rows) * static_cast<size_t>((K + kGsBlk * kGsK - 1) / (kGsBlk * kGsK));
+size_t gemm_slices_expo_ints(int64_t rows, int64_t K) {  // the rows' exponents and the flag `plain`
+    return static_cast<size_t>(rows) * static_cast<size_t>((K + kGsBlk * kGsK - 1) / (kGsBlk * kGsK)) + 1;
 }
 
 // From 512 k: four blocks and the two exponent passes cost less than the FMA kernel's steps at every M
@@ -332,15 +352,20 @@ cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t
     a.part = work;
     a.err = err;
     const unsigned nb = static_cast<unsigned>(a.n_blk);
-    k_exp_max<<<dim3(nb, static_cast<unsigned>((M + 63) / 64)), 256, 0, st>>>(A, lda, M, K, expo);
-    k_exp_max<<<dim3(nb, static_cast<unsigned>((N + 63) / 64)), 256, 0, st>>>(B, ldb, N, K, expo + static_cast<int64_t>(nb) * M);
+    int32_t* expo_b = expo + static_cast<int64_t>(nb) * M;
+    int32_t* plain = expo_b + static_cast<int64_t>(nb) * N;
+    a.plain = plain;
+    e = cudaMemsetAsync(plain, 0, sizeof(int32_t), st);
+    if (e != cudaSuccess) return e;
+    k_exp_max<<<dim3(nb, static_cast<unsigned>((M + 63) / 64)), 256, 0, st>>>(A, lda, M, K, expo, plain);
+    k_exp_max<<<dim3(nb, static_cast<unsigned>((N + 63) / 64)), 256, 0, st>>>(B, ldb, N, K, expo_b, plain);
     const dim3 grid(static_cast<unsigned>((M + kGsM - 1) / kGsM), static_cast<unsigned>((N + kGsN - 1) / kGsN),
                     static_cast<unsigned>(n_split));
     k_gemm_slices<<<grid, kGsThreads, kGsSmem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t mn = static_cast<int64_t>(M) * N;
-    k_slices_reduce<<<static_cast<unsigned>((mn + 255) / 256), 256, 0, st>>>(M, N, n_split, work, C, ldc);
+    k_slices_reduce<<<static_cast<unsigned>((mn + 255) / 256), 256, 0, st>>>(a, n_split, C, ldc);
     return cudaGetLastError();
 }
 

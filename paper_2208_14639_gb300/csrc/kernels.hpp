@@ -425,7 +425,7 @@ cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t
 // M_c + M_c^T, M_c = Phi^T Z_c over the kept points, channels in chunks of `chunk`
 // (ao_channels_per_chunk).  Scratch: phik (nk x nbf), Z and its coefficients (chunk x nk x (nbf +
 // 4), + 1), M (chunk x nbf x nbf) and the product's split-K partials (AoGemm: ao_gemm_work_elems
-// doubles, and the exponents of a product of (chunk + 1) nbf rows over 2 nk points).
+// doubles, and the exponents of a product of (chunk + 1) nbf rows over nk points).
 struct AoGemm {
     double* work;
     size_t work_elems;
