@@ -50,6 +50,23 @@ vv10_status vv10_ctx::ensure(DevBuf& b, size_t bytes, const char* what) {
     return VV10_OK;
 }
 
+// Room for `bytes` in a buffer that a call can do without: no error where there is none, and no
+// allocation while the stream is captured.  The buffer in place is kept until the larger one is there.
+bool vv10_ctx::room(DevBuf& b, size_t bytes, cudaStream_t st) {
+    if (b.bytes >= bytes) return true;
+    if (stream_capturing(st)) return false;
+    if (debug_fail_alloc > 0 && --debug_fail_alloc == 0) return false;
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (b.p) cudaFree(b.p);
+    b.p = p;
+    b.bytes = bytes;
+    return true;
+}
+
 void vv10_ctx::release_all() {
     batch_release();
     DevBuf* bufs[] = {&prep_hist, &prep_offs, &prep_bbox, &prep_small, &orig, &seg, &atom_k,
@@ -413,14 +430,25 @@ vv10_status vv10_ctx::run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_s
     }
     if (!debug_stall && pairsum_sym(mode, fp64)) {
         VV10_TRY(ensure(part, sizeof(double) * nq * static_cast<size_t>(P.nk_pad), "pair sums"));
-        int n_launch = 0;
-        VV10_TRY(ensure(symw, pairsum_sym_work(P.nk_pad, mode, fp64, n_sm, &n_launch), "pair-sum partials"));
-        PhaseScope ph(this, phase, st, n_launch);
-        launches[PH_EP_EPILOGUE] += n_launch;  // the reductions of their partial sums
-        VV10_CUDA(this, launch_pairsum_sym(P, mode, fp64, n_sm, symw.p, static_cast<double*>(part.p), st),
-                  "pair-sum kernel");
-        *n_split_out = 1;
-        return VV10_OK;
+        // Column sums of 1 GB a launch (every offset up to about 210,000 points for E/U/W; beyond, a launch
+        // has hundreds of tile pairs per warp); where that much is not to be had, fewer offsets a
+        // launch, and at last (in a capture too, where nothing can be allocated) the row kernel.
+        size_t last = 0;
+        for (int shift = 30; shift >= 26; shift -= 2) {
+            const size_t cols = size_t(1) << shift;
+            int n_launch = 0;
+            const size_t need = pairsum_sym_work(P.nk_pad, mode, fp64, n_sm, cols, &n_launch);
+            if (need == last || !room(symw, need, st)) {
+                last = need;
+                continue;
+            }
+            PhaseScope ph(this, phase, st, n_launch);
+            launches[PH_EP_EPILOGUE] += n_launch;  // the reductions of their partial sums
+            VV10_CUDA(this, launch_pairsum_sym(P, mode, fp64, n_sm, cols, symw.p, static_cast<double*>(part.p), st),
+                      "pair-sum kernel");
+            *n_split_out = 1;
+            return VV10_OK;
+        }
     }
     PairLaunch cfg;
     const TileChoice tc = tiles_for(mode, fp64);

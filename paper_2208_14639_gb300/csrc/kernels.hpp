@@ -161,12 +161,12 @@ int pairsum_rows64_splits(int64_t nk_pad);
 cudaError_t launch_pairsum_rows64(const PointsDev& p, int mode, double* part, cudaStream_t st);
 
 // The same sums over unordered pairs (pairsum_sym.cu): total[nq][nk_pad] FP64, one split; `work`
-// holds pairsum_sym_work() bytes (n_launch: launches of the pair kernel, each followed
-// by one of its reduction).  pairsum_sym_applies: the
-// sizes at which it is the faster one.
+// holds pairsum_sym_work() bytes: row totals, and column sums of as many tile offsets a launch as
+// col_budget bytes hold (n_launch: launches of the pair kernel, each followed by one of its reduction).
+// pairsum_sym_applies: the sizes at which it is the faster one.
 bool pairsum_sym_applies(int64_t nk, bool fp64);
-size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, int* n_launch);
-cudaError_t launch_pairsum_sym(const PointsDev& p, int mode, bool fp64, int n_sm, void* work,
+size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, size_t col_budget, int* n_launch);
+cudaError_t launch_pairsum_sym(const PointsDev& p, int mode, bool fp64, int n_sm, size_t col_budget, void* work,
                                double* total, cudaStream_t st);
 
 // Batched pair sums (batch.cu): one persistent launch over a task table with an atomic

@@ -479,10 +479,6 @@ int sym_resident(int n_sm) {
     return (n > 0 ? n : 1) * sym_warps<T>() * (n_sm > 0 ? n_sm : 1);
 }
 
-// Scratch of the column sums: a launch covers as many offsets as fit (1 GB: every offset up to
-// about 210,000 points for E/U/W; a launch has hundreds of tile pairs per warp beyond).
-constexpr size_t kSymColBytes = size_t(1) << 30;
-
 struct SymPlan {
     int32_t nb, d_end, offsets;  // tiles; all offsets; offsets per launch
     int32_t warps, split;        // FP64: warps of a launch; FP32: warps per row tile
@@ -502,14 +498,15 @@ struct SymPlan {
     }
 };
 
+// col_budget: bytes of column sums of a launch, which covers as many offsets as fit (at least four).
 template <class T, int MODE, int R>
-SymPlan sym_plan(int64_t nkp, int n_sm) {
+SymPlan sym_plan(int64_t nkp, int n_sm, size_t col_budget) {
     constexpr int TS = 32 * R, NQ = pair_mode_nq(MODE);
     const size_t per_d = sizeof(T) * NQ * static_cast<size_t>(nkp);
     SymPlan P{};
     P.nb = static_cast<int32_t>(nkp / TS);
     P.d_end = P.nb / 2 + 1;
-    int64_t most = static_cast<int64_t>(kSymColBytes / per_d);
+    int64_t most = static_cast<int64_t>(col_budget / per_d);
     if (most < 4) most = 4;
     const int launches = static_cast<int>((P.d_end + most - 1) / most);
     P.offsets = (P.d_end + launches - 1) / launches;
@@ -568,14 +565,14 @@ cudaError_t launch_sym(int64_t nkp, const typename PairRecs<T>::A* ra, const typ
 // Plans (work = null) or runs a mode.  FP32: eight rows per lane (the order of its tile sums).
 // FP64: four, or fewer where more and smaller tiles fill the SMs better.
 template <int MODE>
-cudaError_t sym_mode(const PointsDev* p, int64_t nkp, bool fp64, int n_sm, SymPlan* plan, void* work,
-                     double* total, cudaStream_t st) {
+cudaError_t sym_mode(const PointsDev* p, int64_t nkp, bool fp64, int n_sm, size_t cols, SymPlan* plan,
+                     void* work, double* total, cudaStream_t st) {
     if (!fp64) {
-        *plan = sym_plan<float, MODE, 8>(nkp, n_sm);
+        *plan = sym_plan<float, MODE, 8>(nkp, n_sm, cols);
         return work ? launch_sym<float, MODE, 8>(nkp, p->r32a, p->r32b, *plan, work, total, st) : cudaSuccess;
     }
-    const SymPlan p4 = sym_plan<double, MODE, 4>(nkp, n_sm), p2 = sym_plan<double, MODE, 2>(nkp, n_sm),
-                  p1 = sym_plan<double, MODE, 1>(nkp, n_sm);
+    const SymPlan p4 = sym_plan<double, MODE, 4>(nkp, n_sm, cols), p2 = sym_plan<double, MODE, 2>(nkp, n_sm, cols),
+                  p1 = sym_plan<double, MODE, 1>(nkp, n_sm, cols);
     if (p4.cost <= p2.cost && p4.cost <= p1.cost) {
         *plan = p4;
         return work ? launch_sym<double, MODE, 4>(nkp, p->r64a, p->r64b, p4, work, total, st) : cudaSuccess;
@@ -588,14 +585,14 @@ cudaError_t sym_mode(const PointsDev* p, int64_t nkp, bool fp64, int n_sm, SymPl
     return work ? launch_sym<double, MODE, 1>(nkp, p->r64a, p->r64b, p1, work, total, st) : cudaSuccess;
 }
 
-cudaError_t sym_any(const PointsDev* p, int64_t nkp, int mode, bool fp64, int n_sm, SymPlan* plan,
+cudaError_t sym_any(const PointsDev* p, int64_t nkp, int mode, bool fp64, int n_sm, size_t cols, SymPlan* plan,
                     void* work, double* total, cudaStream_t st) {
     switch (mode) {
-        case MODE_EUW: return sym_mode<MODE_EUW>(p, nkp, fp64, n_sm, plan, work, total, st);
-        case MODE_ABC: return sym_mode<MODE_ABC>(p, nkp, fp64, n_sm, plan, work, total, st);
-        case MODE_GRAD: return sym_mode<MODE_GRAD>(p, nkp, fp64, n_sm, plan, work, total, st);
-        case MODE_EUWABC: return sym_mode<MODE_EUWABC>(p, nkp, fp64, n_sm, plan, work, total, st);
-        default: return sym_mode<MODE_EUWABCG>(p, nkp, fp64, n_sm, plan, work, total, st);
+        case MODE_EUW: return sym_mode<MODE_EUW>(p, nkp, fp64, n_sm, cols, plan, work, total, st);
+        case MODE_ABC: return sym_mode<MODE_ABC>(p, nkp, fp64, n_sm, cols, plan, work, total, st);
+        case MODE_GRAD: return sym_mode<MODE_GRAD>(p, nkp, fp64, n_sm, cols, plan, work, total, st);
+        case MODE_EUWABC: return sym_mode<MODE_EUWABC>(p, nkp, fp64, n_sm, cols, plan, work, total, st);
+        default: return sym_mode<MODE_EUWABCG>(p, nkp, fp64, n_sm, cols, plan, work, total, st);
     }
 }
 
@@ -607,18 +604,18 @@ cudaError_t sym_any(const PointsDev* p, int64_t nkp, int mode, bool fp64, int n_
 // this rule is asked.
 bool pairsum_sym_applies(int64_t nk, bool fp64) { return nk > (fp64 ? 128 : 8192); }
 
-size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, int* n_launch) {
+size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, size_t col_budget, int* n_launch) {
     SymPlan p{};
-    sym_any(nullptr, nk_pad, mode, fp64, n_sm, &p, nullptr, nullptr, nullptr);
+    sym_any(nullptr, nk_pad, mode, fp64, n_sm, col_budget, &p, nullptr, nullptr, nullptr);
     *n_launch = p.launches();
     return p.row_bytes + p.col_bytes;
 }
 
-cudaError_t launch_pairsum_sym(const PointsDev& p, int mode, bool fp64, int n_sm, void* work,
+cudaError_t launch_pairsum_sym(const PointsDev& p, int mode, bool fp64, int n_sm, size_t col_budget, void* work,
                                double* total, cudaStream_t st) {
     if (p.nk == 0) return cudaSuccess;
     SymPlan plan{};
-    return sym_any(&p, p.nk_pad, mode, fp64, n_sm, &plan, work, total, st);
+    return sym_any(&p, p.nk_pad, mode, fp64, n_sm, col_budget, &plan, work, total, st);
 }
 
 }  // namespace vv10

@@ -206,6 +206,7 @@ struct vv10_ctx {
     void set_error(const char* fmt, ...);
     vv10_status cuda_fail(cudaError_t e, const char* where);
     vv10_status ensure(vv10::DevBuf& b, size_t bytes, const char* what);
+    bool room(vv10::DevBuf& b, size_t bytes, cudaStream_t st);
     void release_all();
     vv10_status bind();
     vv10_status check_device_errors(cudaStream_t st);
