@@ -232,7 +232,8 @@ vv10_status vv10_coord_hessian(vv10_handle h, vv10_precision prec, double* E_grg
  *              below rho_cut
  *   prec       VV10_FP64 (VV10_FP64_TC computes the same here), or a mixed mode (FP32
  *              pair arithmetic, FP64 sums)
- * Needs no earlier call other than vv10_prepare_points.  Holds 8 P n_kept bytes of scratch.
+ * Needs no earlier call other than vv10_prepare_points.  Holds 8 P n_kept bytes of scratch; in the
+ * mixed modes about as much again, and where it is to be had 30 MB of one size for every P.
  * Errors: INVALID_ARG, UNSUPPORTED (P too large), OOM, CUDA. */
 vv10_status vv10_weight_response(vv10_handle h, vv10_precision prec, int32_t P,
                                  const double* w_t, double* E_t, double* U_t, double* W_t,

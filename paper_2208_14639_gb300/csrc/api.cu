@@ -72,7 +72,7 @@ void vv10_ctx::release_all() {
     DevBuf* bufs[] = {&prep_hist, &prep_offs, &prep_bbox, &prep_small, &orig, &seg, &atom_k,
                       &soa, &r64a, &r64b, &r32a, &r32b, &r32p, &sumE, &sumU, &sumW, &sumA, &sumB,
                       &sumC, &part, &symw, &eblk, &scal, &tu, &ty, &trt, &tgt, &hacc, &gk,
-                      &tc_uh, &tc_ul, &tc_yh, &tc_yl, &tc16_bh, &tc16_bl, &tc16_small, &o64_sl, &o64_small, &o64_rec, &hvp_fr, &hvp_fg, &nhess, &chpart, &wdir, &wsplit, &ehalf, &aophik, &aoz, &aom, &aogw, &aofa, &ngpart, &dev_err};
+                      &tc_uh, &tc_ul, &tc_yh, &tc_yl, &tc16_bh, &tc16_bl, &tc16_small, &o64_sl, &o64_small, &o64_rec, &tcside, &hvp_fr, &hvp_fg, &nhess, &chpart, &wdir, &wsplit, &wside, &ehalf, &aophik, &aoz, &aom, &aogw, &aofa, &ngpart, &dev_err};
     for (DevBuf* b : bufs) {
         if (b->p) cudaFree(b->p);
         b->p = nullptr;
@@ -925,16 +925,12 @@ vv10_status vv10_weight_response(vv10_handle h, vv10_precision prec, int32_t P,
         weight_tc_groups(P, &ng, &ppad);
         const int32_t rows = ng * ppad;
         const size_t nsplit = static_cast<size_t>(rows) * static_cast<size_t>(Pd.nk_pad);
-        // nsplit is a multiple of 32 x 64: the side outputs after the split stay aligned
-        const size_t side_n = weight_tc_side(Pd.nk, Pd.nk_pad, ng, ppad, h->n_sm);
-        const size_t with_side = 2 * sizeof(float) * nsplit + sizeof(double) * side_n;
-        // without room (or in a capture, where nothing can be allocated) whole tasks are dealt
-        const bool shares = side_n > 0 && (h->wsplit.bytes >= with_side || !stream_capturing(st)) &&
-                            h->ensure(h->wsplit, with_side, "weight direction split") == VV10_OK;
-        if (!shares) VV10_TRY(h->ensure(h->wsplit, 2 * sizeof(float) * nsplit, "weight direction split"));
-        h->set_error("");
+        VV10_TRY(h->ensure(h->wsplit, 2 * sizeof(float) * nsplit, "weight direction split"));
         float* yh = static_cast<float*>(h->wsplit.p);
-        double* side = shares ? reinterpret_cast<double*>(yh + 2 * nsplit) : nullptr;
+        // without room (or in a capture, where nothing can be allocated) whole tasks are dealt
+        double* side = weight_tc_shares(Pd.nk, Pd.nk_pad, ng, h->n_sm) &&
+                               h->room(h->wside, sizeof(double) * side_doubles(h->n_sm), st)
+                           ? static_cast<double*>(h->wside.p) : nullptr;
         PhaseScope ph(h, PH_WEIGHT_RESPONSE, st, side ? 4 : 3);
         VV10_CUDA(h, launch_weight_dirs(Pd, P, w_t, yk, st), "weight directions");
         VV10_CUDA(h, launch_weight_split(yk, P, rows, Pd.nk_pad, yh, yh + nsplit, st),

@@ -910,6 +910,15 @@ static cudaError_t o64_launch(const CUtensorMap* maps, const O64Args& a, int n_s
     return cudaGetLastError();
 }
 
+// Few units per CTA: equal shares of the stages, or the CTAs with one unit more set the time (618
+// units on 152 SMs: 5 rounds for 4.07).  Many: the chunked walk, whose trial tiles stay in L2.  Below
+// 2,048 points a whole unit per CTA: there is little to share, and a few of the smallest systems'
+// elements (where the tiles' 2^-46 shows most) keep their roundings.
+bool hess_o64_shares(int64_t nk, int64_t nk_pad, int n_sm) {
+    static_assert(kO64MaxPpad <= 192, "side_doubles");
+    return 2 * ((nk + 127) / 128) < 16 * static_cast<int64_t>(n_sm) && nk_pad / kO64Kj >= 128;
+}
+
 cudaError_t launch_hess_o64(const PointsDev& p, int32_t Pn, int32_t t0, int64_t acc_P,
                             const void* rec, const void* slices, int64_t slice_stride,
                             int64_t rows, const float* civ, const double* params, int n_sm,
@@ -939,11 +948,7 @@ cudaError_t launch_hess_o64(const PointsDev& p, int32_t Pn, int32_t t0, int64_t 
     const size_t stage_bytes = L.slot_bytes + kO64Kj * kO64RecBytes;
     int64_t chunk = static_cast<int64_t>(kO64ChunkBytes / stage_bytes);
     if (chunk < 64) chunk = 64;
-    // Few units per CTA: equal shares of the stages, or the CTAs with one unit more set the time (618
-    // units on 152 SMs: 5 rounds for 4.07).  Many: the chunked walk, whose trial tiles stay in L2.  Below
-    // 2,048 points a whole unit per CTA: there is little to share, and a few of the smallest systems'
-    // elements (where the tiles' 2^-46 shows most) keep their roundings.
-    a.chunk = a.n_units < 16 * static_cast<int64_t>(n_sm) && a.n_stage >= 128 ? 0 : static_cast<int32_t>(chunk < a.n_stage ? chunk : a.n_stage);
+    a.chunk = side ? 0 : static_cast<int32_t>(chunk < a.n_stage ? chunk : a.n_stage);
     a.side = side;
     a.flush = flush > 0 ? flush : 512;
     a.err = err;

@@ -695,14 +695,12 @@ static int64_t tc_tasks(int64_t nk, int ppad) {
     return (hess_tc_kinds_per_tile(ppad) == 2 ? 1 : 2) * ((nk + 127) / 128);
 }
 
-// Doubles of `side` for equal shares of a launch of Pn trials; 0 where whole tasks are dealt.  Equal shares
-// take 0 to 4 % longer per stage (registers) and a join: milliseconds of the call, whole tasks and shares,
-// 41,000 points P = 54 9.33, 7.12, P = 180 14.46, 14.14; 29,778 points 4.58, 4.27 and 8.48, 7.79; 38,912 points
-// (whole rounds: not taken) 5.96, 5.99 and 11.09, 11.43.
-size_t hess_tc_side(int64_t nk, int64_t nk_pad, int32_t Pn, int flush, int n_sm) {
-    const int ppad = hess_tc_ppad(Pn);
-    if (!shares_pay(tc_tasks(nk, ppad), nk_pad / kTcKj, flush > 0 ? flush : 512, n_sm)) return 0;
-    return static_cast<size_t>(n_sm) * hess_tc_kinds_per_tile(ppad) * static_cast<size_t>(ppad) * 128;
+// Whether a launch of Pn trials deals equal shares.  They take 0 to 4 % longer per stage (registers) and a
+// join: milliseconds of the call, whole tasks and shares, 41,000 points P = 54 9.33, 7.12, P = 180 14.46, 14.14;
+// 29,778 points 4.58, 4.27 and 8.48, 7.79; 38,912 points (whole rounds: not taken) 5.96, 5.99 and 11.09, 11.43.
+bool hess_tc_shares(int64_t nk, int64_t nk_pad, int32_t Pn, int flush, int n_sm) {
+    static_assert(kTcMaxPpad <= 192, "side_doubles");  // and 2 kinds x 64
+    return shares_pay(tc_tasks(nk, hess_tc_ppad(Pn)), nk_pad / kTcKj, flush > 0 ? flush : 512, n_sm);
 }
 
 // Contract the trials [t0, t0 + Pn) (Pn <= 192) of one system; split arrays have `rows` rows.

@@ -150,26 +150,23 @@ vv10_status vv10_ctx::tc_contract(int32_t Pn, int cap, cudaStream_t st) {
                "trial split");
     }
     const size_t ab = sizeof(double) * 2 * static_cast<size_t>(Pn) * P.nk_pad;
-    // equal shares of the stages need a side output after the partials; without room (or in a
-    // capture, where nothing can be allocated), whole tasks
+    H_TRY(ensure(hacc, ab, "contraction partials"));
+    // equal shares of the stages need side outputs; without room (or in a capture, where nothing can be
+    // allocated), whole tasks
     auto group = [&](int g) { return std::min(pg, Pn - g * pg); };
-    auto side_n = [&](int g) { return hess_tc_side(P.nk, P.nk_pad, group(g), tc_flush, n_sm); };
-    const size_t sd = sizeof(double) * std::max(side_n(0), side_n(ng - 1));
-    const bool shares = sd > 0 && (hacc.bytes >= ab + sd || !stream_capturing(st)) &&
-                        ensure(hacc, ab + sd, "contraction partials") == VV10_OK;
-    if (!shares) H_TRY(ensure(hacc, ab, "contraction partials"));
-    set_error("");
-    double* side = shares ? reinterpret_cast<double*>(static_cast<char*>(hacc.p) + ab) : nullptr;
+    auto shares = [&](int g) { return hess_tc_shares(P.nk, P.nk_pad, group(g), tc_flush, n_sm); };
+    double* side = (shares(0) || shares(ng - 1)) && room(tcside, sizeof(double) * side_doubles(n_sm), st)
+                       ? static_cast<double*>(tcside.p) : nullptr;
     H_CUDA(cudaMemsetAsync(hacc.p, 0, ab, st), "zero contraction partials");
     int launches = ng;
-    for (int g = 0; g < ng; ++g) launches += side && side_n(g) > 0;
+    for (int g = 0; g < ng; ++g) launches += side && shares(g);
     PhaseScope ph(this, PH_CONTRACT_TC, st, launches);
     for (int g = 0; g < ng; ++g) {
         const int t0 = g * pg, pn = group(g);
         H_CUDA(launch_hess_tc(P, pn, t0, Pn, static_cast<float*>(tc_uh.p),
                               static_cast<float*>(tc_ul.p), static_cast<float*>(tc_yh.p),
                               static_cast<float*>(tc_yl.p), rows, n_sm, tc_flush,
-                              static_cast<double*>(hacc.p), side_n(g) > 0 ? side : nullptr,
+                              static_cast<double*>(hacc.p), shares(g) ? side : nullptr,
                               static_cast<int*>(dev_err.p), st),
                "tensor-core contraction");
     }
@@ -244,8 +241,9 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
                "FP64 trial slices");
     }
     const size_t ab = sizeof(double) * 2 * static_cast<size_t>(Pn) * P.nk_pad;
-    // side outputs for the widest launch, whatever pg: the buffer never has to grow for fewer trials
-    H_TRY(ensure(hacc, ab + sizeof(double) * 128 * static_cast<size_t>(cap) * n_sm, "contraction partials"));
+    H_TRY(ensure(hacc, ab, "contraction partials"));
+    double* side = hess_o64_shares(P.nk, P.nk_pad, n_sm) && room(tcside, sizeof(double) * side_doubles(n_sm), st)
+                       ? static_cast<double*>(tcside.p) : nullptr;  // without room whole units
     H_CUDA(cudaMemsetAsync(hacc.p, 0, ab, st), "zero contraction partials");
     const int64_t civ_group = civ_n / ng;
     PhaseScope ph(this, PH_CONTRACT_TC, st, ng);
@@ -253,8 +251,7 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
         const int t0 = g * pg;
         const int pn = (Pn - t0 < pg) ? Pn - t0 : pg;
         H_CUDA(launch_hess_o64(P, pn, t0, Pn, o64_rec.p, o64_sl.p, stride, rows, civ + g * civ_group,
-                               params, n_sm, tc_flush, pg, static_cast<double*>(hacc.p),
-                               static_cast<double*>(hacc.p) + ab / sizeof(double),
+                               params, n_sm, tc_flush, pg, static_cast<double*>(hacc.p), side,
                                static_cast<int*>(dev_err.p), st),
                "FP64 tensor-core contraction");
     }

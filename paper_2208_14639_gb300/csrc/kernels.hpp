@@ -254,8 +254,11 @@ inline bool shares_pay(int64_t n_tasks, int64_t n_stage, int64_t flush, int64_t 
     }
     return 20 * worst <= 19 * whole;
 }
-// `side`: hess_tc_side doubles, or null (whole tasks are dealt to the CTAs).
-size_t hess_tc_side(int64_t nk, int64_t nk_pad, int32_t Pn, int flush, int n_sm);
+// Side outputs of CTAs whose share begins inside a task: one size for every launch of the contractions
+// and the weight-derivative sums, so that the buffer is allocated once and never moves.
+inline size_t side_doubles(int n_sm) { return static_cast<size_t>(n_sm) * 192 * 128; }
+// Whether a launch of Pn trials deals equal shares; `side`: side_doubles(n_sm), or null (whole tasks).
+bool hess_tc_shares(int64_t nk, int64_t nk_pad, int32_t Pn, int flush, int n_sm);
 cudaError_t launch_hess_tc(const PointsDev& p, int32_t Pn, int32_t t0, int64_t acc_P,
                            const float* uh, const float* ul, const float* yh, const float* yl,
                            int64_t rows, int n_sm, int flush, double* acc, double* side, int* err,
@@ -300,7 +303,8 @@ cudaError_t launch_hess_f16(const PointsDev& p, int32_t Pn, int32_t t0, int64_t 
 // inverses civ [group][nk_pad / 16][hess_o64_ppad(pg)] for trial groups of pg <=
 // hess_o64_max_group() (hess_o64_civ_floats floats).  launch_hess_o64 contracts the trials [t0, t0 + Pn), Pn <= pg,
 // with `civ` pointing at their group's block, into acc [2][acc_P][nk_pad] (zeroed by the
-// caller); side: n_sm x Pn x 128 doubles of scratch.
+// caller).  hess_o64_shares: whether equal shares are dealt; side: side_doubles(n_sm), or null (whole units).
+bool hess_o64_shares(int64_t nk, int64_t nk_pad, int n_sm);
 int hess_o64_max_group();
 int hess_o64_ppad(int32_t pg);
 int hess_o64_slices();
@@ -387,8 +391,8 @@ cudaError_t launch_weight_response(const PointsDev& p, bool fp64, int32_t Pn, co
 void weight_tc_groups(int32_t P, int* n_groups, int* ppad);
 cudaError_t launch_weight_split(const double* yk, int32_t Pn, int32_t rows, int64_t nk_pad,
                                 float* yh, float* yl, cudaStream_t st);
-// `side`: weight_tc_side doubles, or null (whole tasks are dealt to the CTAs).
-size_t weight_tc_side(int64_t nk, int64_t nk_pad, int n_groups, int ppad, int n_sm);
+// Whether equal shares are dealt; `side`: side_doubles(n_sm), or null (whole tasks).
+bool weight_tc_shares(int64_t nk, int64_t nk_pad, int n_groups, int n_sm);
 cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, const float* yl,
                              int32_t rows, double* E, double* U, double* W, int n_sm, double* side, int* err,
                              cudaStream_t st);

@@ -148,6 +148,7 @@ struct vv10_ctx {
     vv10::DevBuf o64_sl;            // FP64-accurate contraction: FP16 trial slice arrays
     vv10::DevBuf o64_small;         // their factors and y balance
     vv10::DevBuf o64_rec;           // and the points' FP32-pair column records
+    vv10::DevBuf tcside;            // side outputs of the contractions' equal shares
     vv10::DevBuf hvp_fr, hvp_fg;    // Hessian-vector product: the contraction's outputs
 
     // coordinate scratch
@@ -155,6 +156,7 @@ struct vv10_ctx {
     vv10::DevBuf chpart;  // per-CTA partials of the grid-grid Hessian blocks
     vv10::DevBuf wdir;    // weight directions in kept order (weight-derivative sums)
     vv10::DevBuf wsplit;  // their TF32 hi / FP32 lo split (tensor-core path)
+    vv10::DevBuf wside;   // side outputs of their equal shares
     vv10::DevBuf ehalf;   // per-CTA totals of the energy-only kernel
     vv10::DevBuf aophik, aoz, aom;  // AO assembly: gathered phi, Z, GEMM results
     vv10::DevBuf aogw;              // AO assembly: split-K partials of its FP64 products

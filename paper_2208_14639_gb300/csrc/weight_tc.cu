@@ -525,12 +525,11 @@ cudaError_t launch_weight_split(const double* yk, int32_t Pn, int32_t rows, int6
     return cudaGetLastError();
 }
 
-// Doubles of `side` for equal shares of the stages; 0 where whole tasks are dealt.  Equal shares take about
-// 2 % longer per stage (registers) and a join: milliseconds of the call, whole tasks and shares, 41,000
+// Whether equal shares of the stages are dealt.  They take about 2 % longer per stage (registers) and a join: milliseconds of the call, whole tasks and shares, 41,000
 // points P = 18 7.21, 5.32, P = 54 7.80, 5.82; 38,912 points (two whole rounds) 4.57, 4.64 and 4.91, 5.02.
-size_t weight_tc_side(int64_t nk, int64_t nk_pad, int n_groups, int ppad, int n_sm) {
-    if (!shares_pay(static_cast<int64_t>(n_groups) * ((nk + 127) / 128), nk_pad / kWtKj, kWtFlush, n_sm)) return 0;
-    return static_cast<size_t>(n_sm) * kWtKinds * static_cast<size_t>(ppad) * 128;
+bool weight_tc_shares(int64_t nk, int64_t nk_pad, int n_groups, int n_sm) {
+    static_assert(kWtKinds * kWtMaxPpad <= 192, "side_doubles");
+    return shares_pay(static_cast<int64_t>(n_groups) * ((nk + 127) / 128), nk_pad / kWtKj, kWtFlush, n_sm);
 }
 
 cudaError_t launch_weight_tc(const PointsDev& p, int32_t Pn, const float* yh, const float* yl,
