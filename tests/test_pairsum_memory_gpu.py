@@ -87,3 +87,28 @@ def test_captured_without_scratch(dev, prec, n):
         assert torch.equal(vr, vr_rows) and torch.equal(vg, vg_rows)
     finally:
         eng.close()
+
+
+@pytest.mark.parametrize("first,prec,later", [(5000, FP64, 4000), (4000, MIXED, 4000)], ids=["smaller", "fp64"])
+def test_graph_survives_a_small_fp64_system(dev, first, prec, later):
+    """The small FP64 kernel's partials, larger than a 5,000-point system's or an FP32 call's, leave the
+    buffer in place that a captured call uses; prepared again as at the capture, it replays its bits."""
+    T = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev, torch.float64)
+    a, b = synth.random_points(first, seed=1), synth.random_points(later, seed=2)
+    da, db = ([T(x) for x in (g.coords, g.weights, g.rho, g.grad_rho)] for g in (a, b))
+    eng = vv10.VV10(0)
+    try:
+        assert eng.prepare(*da) == first
+        _, vr_ref, vg_ref = eng.energy_potential(prec)
+        vr, vg = torch.zeros_like(vr_ref), torch.zeros_like(vg_ref)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            vv10.vv10_energy_potential(eng.h, prec, vr, vg, torch.cuda.current_stream(), False)
+        eng.prepare(*db)
+        eng.energy_potential(FP64)
+        eng.prepare(*da)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(vr, vr_ref) and torch.equal(vg, vg_ref)
+    finally:
+        eng.close()
