@@ -196,7 +196,7 @@ cudaError_t fma_product(const AoGemm& g, int M, int N, int64_t K, const double* 
     const size_t per = static_cast<size_t>(M) * static_cast<size_t>(N);
     const int cap = static_cast<int>(g.work_elems / (per > 0 ? per : 1));
     s = s < cap ? s : (cap > 0 ? cap : 1);
-    return launch_gemm_abt(M, N, K, A, M, B, N, C, M, g.work, s, st);
+    return launch_gemm_abt(M, N, K, A, M, B, N, C, M, g.work, s, g.launched, st);
 }
 
 // The same on the tensor cores unless it is short.
@@ -204,7 +204,8 @@ cudaError_t ao_product(const AoGemm& g, int M, int N, int64_t K, const double* A
                        double* C, cudaStream_t st) {
     if (gemm_slices_applies(K))
         return launch_gemm_slices(M, N, K, A, M, B, N, C, M, g.work,
-                                  gemm_slices_splits(M, N, K, g.n_sm, g.work_elems), g.expo, g.err, st);
+                                  gemm_slices_splits(M, N, K, g.n_sm, g.work_elems), g.expo, g.launched, g.err,
+                                  st);
     return fma_product(g, M, N, K, A, B, C, st);
 }
 
@@ -221,6 +222,7 @@ cudaError_t assemble_chunks(const PointsDev& p, const AoGemm& g, int32_t nbf, in
     AoCoef* coef = reinterpret_cast<AoCoef*>(Z + ((p.nk * nbf * chunk + 1) & ~int64_t(1)));
     for (int32_t c0 = 0; c0 < n_ch; c0 += static_cast<int32_t>(chunk)) {
         const int32_t nc = static_cast<int32_t>(n_ch - c0 < chunk ? n_ch - c0 : chunk);
+        *g.launched += 3;  // coefficients, Z, symmetrisation
         make_coef(c0, nc, coef);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -252,6 +254,7 @@ cudaError_t launch_ao_assemble(const PointsDev& p, const AoGemm& g, int32_t nbf,
     if (p.nk == 0) return cudaMemsetAsync(out, 0, sizeof(double) * nn * n_ch, st);
     const int64_t ne = p.nk * nbf;
     const unsigned gx = static_cast<unsigned>((ne + 255) / 256);
+    *g.launched += 1;
     k_ao_gather<<<gx, 256, 0, st>>>(p, nbf, phi, phik);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -272,6 +275,7 @@ cudaError_t launch_fock_derivative(const PointsDev& p, const AoGemm& g, const Fo
     const int64_t ne = p.nk * nbf;
     const unsigned gx = static_cast<unsigned>((ne + 255) / 256);
     const unsigned gn = static_cast<unsigned>((nn + 255) / 256);
+    *g.launched += 1;
     k_ao_gather<<<gx, 256, 0, st>>>(p, nbf, in.phi, phik);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -291,10 +295,12 @@ cudaError_t launch_fock_derivative(const PointsDev& p, const AoGemm& g, const Fo
     double* L = LR + 2 * ne;
     double* Kall = K2;
     double* KA = K2 + nn;
+    *g.launched += 1;
     k_fa_right<<<gx, 256, 0, st>>>(p, in, R);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     for (int c = 0; c < 3; ++c) {
+        *g.launched += 1 + p.n_atom;  // the left factor, each atom's update
         k_fa_left<<<gx, 256, 0, st>>>(p, in, c, L);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -1008,9 +1008,10 @@ static vv10_status ao_assemble(vv10_handle h, int32_t nbf, const double* phi, co
     VV10_TRY(h->ensure(h->aom, sizeof(double) * static_cast<size_t>(nbf) * nbf * chunk, "assembly products"));
     const size_t gw = ao_gemm_work_elems(nbf, chunk, h->n_sm);
     VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), P.nk), "assembly product partials"));
+    int launched = 0;
     const AoGemm g{static_cast<double*>(h->aogw.p), gw, reinterpret_cast<int32_t*>(static_cast<double*>(h->aogw.p) + gw),
-                   h->n_sm, static_cast<int*>(h->dev_err.p)};
-    PhaseScope ph(h, PH_AO_ASSEMBLY, st, P.nk > 0 ? 1 + 4 * static_cast<int>((n_ch + chunk - 1) / chunk) : 0);
+                   h->n_sm, &launched, static_cast<int*>(h->dev_err.p)};
+    CountedPhase ph(h, PH_AO_ASSEMBLY, st, &launched);
     VV10_CUDA(h, launch_ao_assemble(P, g, nbf, phi, dphi, n_ch, s, fg, vg, gt, chunk,
                                     static_cast<double*>(h->aophik.p), static_cast<double*>(h->aoz.p),
                                     static_cast<double*>(h->aom.p), out, st),
@@ -1093,8 +1094,9 @@ vv10_status vv10_fock_derivative(vv10_handle h, int32_t nbf, const double* phi,
     VV10_TRY(h->ensure(h->aofa, sizeof(double) * (4 * nk * nbf + 2 * nn), "basis-derivative factors"));
     const size_t gw = ao_gemm_work_elems(nbf, chunk, h->n_sm);
     VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), P.nk), "assembly product partials"));
+    int launched = 0;
     const AoGemm g{static_cast<double*>(h->aogw.p), gw, reinterpret_cast<int32_t*>(static_cast<double*>(h->aogw.p) + gw),
-                   h->n_sm, static_cast<int*>(h->dev_err.p)};
+                   h->n_sm, &launched, static_cast<int*>(h->dev_err.p)};
     std::vector<int64_t> seg(static_cast<size_t>(P.n_atom) + 1);
     VV10_CUDA(h, cudaMemcpyAsync(seg.data(), P.seg, sizeof(int64_t) * seg.size(),
                                  cudaMemcpyDeviceToHost, st), "atom segments");
@@ -1102,12 +1104,7 @@ vv10_status vv10_fock_derivative(vv10_handle h, int32_t nbf, const double* phi,
     FockDerivIn in{nbf, phi, grad_phi, hess_phi, bf_atom, vrho, vgamma, f_rho_a, f_gamma_a,
                    grad_rho_a, w_a, E_w, U_w, W_w, EUW_gr};
     double* fa = static_cast<double*>(h->aofa.p);
-    // launches: gather, right factor, per chunk (Z, product, its split sum, symmetrisation),
-    // per direction c (left factor, product + split sum, per atom product + split sum and
-    // the basis-derivative update)
-    const int n_launch =
-        P.nk > 0 ? 2 + 4 * static_cast<int>((n_dir + chunk - 1) / chunk) + 3 * (3 + 3 * P.n_atom) : 0;
-    PhaseScope ph(h, PH_AO_ASSEMBLY, st, n_launch);
+    CountedPhase ph(h, PH_AO_ASSEMBLY, st, &launched);
     VV10_CUDA(h, launch_fock_derivative(P, g, in, seg.data(), chunk,
                                         static_cast<double*>(h->aophik.p),
                                         static_cast<double*>(h->aoz.p),

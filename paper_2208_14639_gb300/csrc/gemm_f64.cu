@@ -100,7 +100,7 @@ int gemm_abt_splits(int M, int N, int64_t K, int n_sm) {
 
 cudaError_t launch_gemm_abt(int M, int N, int64_t K, const double* A, int64_t lda, const double* B,
                             int64_t ldb, double* C, int64_t ldc, double* work, int n_split,
-                            cudaStream_t st) {
+                            int* launched, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (K <= 0) {
         for (int n = 0; n < N; ++n) {
@@ -115,6 +115,7 @@ cudaError_t launch_gemm_abt(int M, int N, int64_t K, const double* A, int64_t ld
     n_split = static_cast<int>((K + kps - 1) / kps);
     const dim3 grid(static_cast<unsigned>((M + kGT - 1) / kGT), static_cast<unsigned>((N + kGT - 1) / kGT),
                     static_cast<unsigned>(n_split));
+    *launched += n_split == 1 ? 1 : 2;
     if (n_split == 1) {
         k_gemm_abt<<<grid, kGThreads, 0, st>>>(M, N, K, kps, A, lda, B, ldb, C, ldc, 0);
         return cudaGetLastError();

@@ -332,7 +332,7 @@ int gemm_slices_splits(int M, int N, int64_t K, int n_sm, size_t work_elems) {
 
 cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t lda, const double* B,
                                int64_t ldb, double* C, int64_t ldc, double* work, int n_split,
-                               int32_t* expo, int* err, cudaStream_t st) {
+                               int32_t* expo, int* launched, int* err, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(k_gemm_slices, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kGsSmem));
     if (e != cudaSuccess) return e;
@@ -355,6 +355,7 @@ cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t
     int32_t* expo_b = expo + static_cast<int64_t>(nb) * M;
     int32_t* plain = expo_b + static_cast<int64_t>(nb) * N;
     a.plain = plain;
+    *launched += 4;
     e = cudaMemsetAsync(plain, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     k_exp_max<<<dim3(nb, static_cast<unsigned>((M + 63) / 64)), 256, 0, st>>>(A, lda, M, K, expo, plain);

@@ -233,7 +233,7 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
     double* params = reinterpret_cast<double*>(sm + 16);
     float* civ = reinterpret_cast<float*>(sm + 32);
     {
-        PhaseScope ph(this, PH_TRIAL_PREP, st, 5);
+        PhaseScope ph(this, PH_TRIAL_PREP, st, 4);
         H_CUDA(launch_o64_prep(P, static_cast<double*>(tu.p), static_cast<double*>(ty.p), Pn,
                                static_cast<int32_t>(rows), pg, o64_rec.p,
                                reinterpret_cast<unsigned long long*>(sm), params, o64_sl.p, stride,
@@ -246,7 +246,7 @@ vv10_status vv10_ctx::o64_contract(int32_t Pn, cudaStream_t st) {
                        ? static_cast<double*>(tcside.p) : nullptr;  // without room whole units
     H_CUDA(cudaMemsetAsync(hacc.p, 0, ab, st), "zero contraction partials");
     const int64_t civ_group = civ_n / ng;
-    PhaseScope ph(this, PH_CONTRACT_TC, st, ng);
+    PhaseScope ph(this, PH_CONTRACT_TC, st, side ? 2 * ng : ng);  // with the shares' joins
     for (int g = 0; g < ng; ++g) {
         const int t0 = g * pg;
         const int pn = (Pn - t0 < pg) ? Pn - t0 : pg;

@@ -411,11 +411,11 @@ cudaError_t launch_energy_half(const PointsDev& p, bool fp64, int grid, double* 
 
 // FP64 C = A B^T (gemm_f64.cu): A M x K, B N x K with k slowest (column k at A + k lda), C
 // M x N column-major; the K range split n_split ways (gemm_abt_splits), partials in work
-// (n_split x M x N doubles) summed in a fixed order.
+// (n_split x M x N doubles) summed in a fixed order.  *launched grows by the kernels launched.
 int gemm_abt_splits(int M, int N, int64_t K, int n_sm);
 cudaError_t launch_gemm_abt(int M, int N, int64_t K, const double* A, int64_t lda, const double* B,
                             int64_t ldb, double* C, int64_t ldc, double* work, int n_split,
-                            cudaStream_t st);
+                            int* launched, cudaStream_t st);
 
 // The same product on the tensor cores, as exact integer slice products (gemm_slices.cu); work as
 // above, expo: gemm_slices_expo_ints(M + N, K), err: the device error word.
@@ -425,7 +425,7 @@ bool gemm_slices_applies(int64_t K);
 int gemm_slices_splits(int M, int N, int64_t K, int n_sm, size_t work_elems);
 cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t lda, const double* B,
                                int64_t ldb, double* C, int64_t ldc, double* work, int n_split,
-                               int32_t* expo, int* err, cudaStream_t st);
+                               int32_t* expo, int* launched, int* err, cudaStream_t st);
 
 // AO-side assembly (Sec. II.A Fock matrix, Sec. II.B contracted orbital Hessian): out[c] =
 // M_c + M_c^T, M_c = Phi^T Z_c over the kept points, channels in chunks of `chunk`
@@ -437,6 +437,7 @@ struct AoGemm {
     size_t work_elems;
     int32_t* expo;
     int n_sm;
+    int* launched;  // grows by the kernels that the assembly launches
     int* err;
 };
 size_t ao_gemm_work_elems(int32_t nbf, int64_t chunk, int n_sm);

@@ -245,4 +245,10 @@ struct PhaseScope {
     }
     ~PhaseScope() { h->phase_end(&rec, st, n); }
 };
+// The same with a count that the launches themselves keep.
+struct CountedPhase : PhaseScope {
+    const int* launched;
+    CountedPhase(vv10_ctx* h_, int phase, cudaStream_t s, const int* l) : PhaseScope(h_, phase, s, 0), launched(l) {}
+    ~CountedPhase() { n = *launched; }
+};
 }  // namespace vv10
