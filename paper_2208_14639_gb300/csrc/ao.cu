@@ -179,8 +179,9 @@ size_t ao_gemm_work_elems(int32_t nbf, int64_t chunk, int n_sm) {
     return big > small ? big : small;
 }
 
+// Channels whose Z fits max_bytes; their coefficients, 4 / nbf of it, add a quarter at most.
 int64_t ao_channels_per_chunk(int64_t nk, int32_t nbf, int32_t n_ch, size_t max_bytes) {
-    const size_t per = sizeof(double) * static_cast<size_t>(nk > 0 ? nk : 1) * static_cast<size_t>(nbf);
+    const size_t per = sizeof(double) * static_cast<size_t>(nk > 0 ? nk : 1) * static_cast<size_t>(nbf < 16 ? 16 : nbf);
     int64_t c = static_cast<int64_t>(max_bytes / per);
     if (c < 1) c = 1;
     return c < n_ch ? c : n_ch;
