@@ -84,17 +84,20 @@ __device__ __forceinline__ float rcp_refined(float x) {
     return fmaf(r, e, r);
 }
 __device__ __forceinline__ float recip(float x) { return rcp_refined(x); }
-// Reciprocal in FP64: the hardware's approximation (about 20 bits, FP32-rate unit) and one
-// third-order step r' = r (1 + e + e^2), e = 1 - x r, whose remainder e^3 is below the rounding:
-// three FP64 operations on GB300's narrow pipe, no branch, within one unit in the last place.
-// An infinite or NaN x keeps the approximation's 0 or NaN (the step would form 0 x inf).
+// Reciprocal in FP64: the hardware's approximation (about 20 bits, FP32-rate unit) and one step of the
+// third-order iteration r' = r (1 + e + e^2), e = 1 - x r (Householder's method for 1/x, of order two),
+// whose remainder e^3 is below the rounding: three FP64 operations on GB300's narrow pipe, no branch,
+// within one unit in the last place for 2^-1022 <= |x| < 2^1022.  Where the approximation is 0 or not
+// finite it is the result (the step would form 0 x inf): 1/0 and 1/inf as the divide gives them, 0 from
+// 2^1022 on, and an infinity for subnormal x.
 __device__ __forceinline__ double recip(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     double e = __fma_rn(-x, r, 1.0);
     e = __fma_rn(e, e, e);
     const double y = __fma_rn(r, e, r);
-    return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000 ? r : y;
+    const unsigned ex = static_cast<unsigned>(__double2hiint(r)) & 0x7ff00000u;
+    return ex - 0x00100000u < 0x7fe00000u ? y : r;
 }
 
 // Packed per-point records of the pair kernels for arithmetic type T (PointsDev r32a/r32b or
