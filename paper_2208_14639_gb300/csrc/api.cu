@@ -422,10 +422,10 @@ vv10_status vv10_ctx::run_pairsum(int mode, bool fp64, cudaStream_t st, int* n_s
                       : (mode == MODE_ABC ? PH_PAIR_ABC : PH_PAIR_GRAD);
     // The small FP64 kernel's partials are larger than those of systems beyond it: room for them from the
     // start, so that a smaller system, or FP64 after FP32, does not move the buffer.
-    if (fp64 || pairsum_rows64_applies(P.nk)) room(part, pairsum_rows64_part(P.nk_pad), st);
+    if (fp64 || pairsum_rows64_applies(P.nk)) room(part, pairsum_rows64_part(nq, P.nk_pad), st);
     const int ns64 = pairsum_rows64_splits(P.nk_pad);
     if (!debug_stall && fp64 && pairsum_rows64_applies(P.nk) && !pairsum_fixed(mode, fp64) &&
-        room(part, sizeof(double) * nq * static_cast<size_t>(ns64) * P.nk_pad, st)) {
+        part.bytes >= sizeof(double) * nq * static_cast<size_t>(ns64) * P.nk_pad) {
         PhaseScope ph(this, phase, st, 1);
         VV10_CUDA(this, launch_pairsum_rows64(P, mode, static_cast<double*>(part.p), st), "pair-sum kernel");
         *n_split_out = ns64;

@@ -156,9 +156,9 @@ cudaError_t launch_pairsum(const PointsDev& p, int mode, bool fp64, const PairLa
 int pairsum_default_split(const PointsDev& p, int mode, bool fp64, int rows_per_thread, int n_sm);
 
 // FP64 sums of a small system: part[nq][pairsum_rows64_splits(nk_pad)][nk_pad].  pairsum_rows64_part: bytes
-// with which no such system of at most nk points, in any mode, needs a larger part (38 MB from 4,096).
+// with which no such system of at most nk points needs a larger part for nq sums (three: 13 MB from 4,096).
 bool pairsum_rows64_applies(int64_t nk);
-size_t pairsum_rows64_part(int64_t nk_pad);
+size_t pairsum_rows64_part(int nq, int64_t nk_pad);
 int pairsum_rows64_splits(int64_t nk_pad);
 cudaError_t launch_pairsum_rows64(const PointsDev& p, int mode, double* part, cudaStream_t st);
 

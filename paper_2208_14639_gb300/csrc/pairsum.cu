@@ -196,10 +196,10 @@ static cudaError_t launch_mode(const PointsDev& p, bool fp64, const PairLaunch& 
 constexpr int64_t kRows64Max = 4096;
 bool pairsum_rows64_applies(int64_t nk) { return nk <= kRows64Max; }
 int pairsum_rows64_splits(int64_t nk_pad) { return static_cast<int>(nk_pad / kRows64J); }
-size_t pairsum_rows64_part(int64_t nk_pad) {
+size_t pairsum_rows64_part(int nq, int64_t nk_pad) {
     static_assert(kRows64Max % kJTile == 0, "padded sizes up to kRows64Max");
     const size_t n = static_cast<size_t>(nk_pad < kRows64Max ? nk_pad : kRows64Max);
-    return sizeof(double) * pair_mode_nq(MODE_EUWABCG) * (n / kRows64J) * n;
+    return sizeof(double) * nq * (n / kRows64J) * n;
 }
 
 cudaError_t launch_pairsum_rows64(const PointsDev& p, int mode, double* part, cudaStream_t st) {
