@@ -246,8 +246,13 @@ vv10_status vv10_weight_response(vv10_handle h, vv10_precision prec, int32_t P,
  *   G^t_mu_nu = sum_i w_i [f^{rho,t}_i phi_mu phi_nu
  *                          + 2 (f^{gamma,t}_i grad rho_i + f^gamma_i grad rho^t_i)
  *                            . (phi_nu grad phi_mu + phi_mu grad phi_nu)]
- * over the points kept at vv10_prepare_points (w and grad rho as prepared), to FP64 accuracy (one
- * product over the points, the trials side by side).  For rho = sum P_mu_nu phi_mu phi_nu, F_mu_nu = dE/dP_mu_nu
+ * over the points kept at vv10_prepare_points (w and grad rho as prepared), to FP64 accuracy in norm
+ * (one product over the points, the trials side by side).  From 512 kept points on the product's factors
+ * phi_mu and Z_nu (the weighted combination of phi_nu and grad phi_nu) are cut relative to their largest
+ * value in each block of 128 consecutive kept points: besides FP64 rounding an element is off by
+ * about 2^-56 of the sum of max |phi_mu| max |Z_nu| over the blocks.  In grid order (neighbouring points
+ * of like magnitude) that is below the rounding; with core functions and an atom's points in random
+ * order, elements have been off by up to 1e-12 of their sum of absolute terms.  For rho = sum P_mu_nu phi_mu phi_nu, F_mu_nu = dE/dP_mu_nu
  * and G^t = dF along P^t.
  *   nbf          number of basis functions, 1 <= nbf <= VV10_MAX_BASIS
  *   phi          n x nbf device in, phi_mu at point i at phi[i nbf + mu] (caller order)
@@ -293,7 +298,8 @@ vv10_status vv10_nuclear_gradient(vv10_handle h, int32_t P, const double* rho_t,
  * with B_mu_nu = grad(phi_mu phi_nu), s^a = f^{rho,a} + E^{aw} + E^{a,gr} + rho (kappa' (U^{aw} +
  * U^{a,gr}) + omega_rho (W^{aw} + W^{a,gr})), t^a = f^{gamma,a} + rho omega_gamma (W^{aw} +
  * W^{a,gr}) and d_a phi_mu(i) = ([A owns point i] - [A is the centre of mu]) d phi_mu / d x_c.
- * Sums over the points kept at vv10_prepare_points, to FP64 accuracy.
+ * Sums over the points kept at vv10_prepare_points, to FP64 accuracy, the terms without d_a phi as
+ * vv10_orbital_hessian's.
  * Needs atom_of_point at prepare time (n_atom >= 1, else INVALID_ARG).
  *   nbf, phi, grad_phi   as for vv10_fock_matrix
  *   hess_phi             n x nbf x 3 x 3 device in: second derivatives of phi_mu at point i
