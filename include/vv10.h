@@ -66,7 +66,8 @@ typedef enum {
                                leading products the tensor cores sum exactly in FP32, up to
                                64 trials a launch; results agree with VV10_FP64 to
                                ~1e-11 relative in norm, each element to ~1e-10 of its size
-                               (the double-FP32 tiles carry ~46 bits).  Single systems only:
+                               and the rms (the double-FP32 tiles carry ~46 bits: single
+                               elements to 3e-10, a typical worst one 3e-11).  Single systems only:
                                the batched contraction returns VV10_ERR_UNSUPPORTED.       */
 } vv10_precision;
 
