@@ -135,7 +135,7 @@ vv10_status vv10_prepare_points(vv10_handle h, int64_t n, const double* xyz, con
  *   vrho      n device out, f^rho (may be NULL)
  *   vgamma    n device out, f^gamma (may be NULL)
  * Caches E_i, U_i, W_i in the handle for vv10_hessian_contract / vv10_weight_grad.
- * Scratch of the pair sums, here and in every call that forms them: above 8,192 kept points (FP64:
+ * Scratch of the pair sums, here and in every call that forms them: above 10,752 kept points (FP64:
  * 4,096) column sums of at most 1 GB and some hundred MB of row totals (131,008 points, three sums,
  * mixed: 0.5 GB in all), which the handle keeps.  Where that is not to be had less is taken, and at
  * the least (also in a stream capture that finds no scratch in place) a kernel that needs a few ten MB.

@@ -598,11 +598,13 @@ cudaError_t sym_any(const PointsDev* p, int64_t nkp, int mode, bool fp64, int n_
 
 }  // namespace
 
-// FP32: a tile pair is one warp's work, so below some thirty tiles the warps are too few (7,211
-// points E/U/W 0.114 ms against 0.108 row by row, 11,932 points 0.151 against 0.19).  FP64: the
-// tiles shrink with the system; the smallest systems take pairsum.cu's small FP64 kernel before
-// this rule is asked.
-bool pairsum_sym_applies(int64_t nk, bool fp64) { return nk > (fp64 ? 128 : 8192); }
+// FP32: a tile pair is one warp's work, so below some forty tiles the warps are too few.  Calls of three,
+// six and nine sums, microseconds row by row and here: 8,684 points 104, 128, 200 and 103, 134, 209; 10,732
+// points 135, 176, 259 and 135, 192, 285; 10,988 points 164, 233, 304 and 136, 190, 285; 15,852 points 266,
+// 354, 468 and 224, 321, 462.  (Both kernels' times are stairs: at 12,780 to 13,036 points six sums are 12 %,
+// and up to 15,340 nine sums 8 to 11 %, slower here.)  FP64: the tiles shrink with the system; the smallest
+// systems take pairsum.cu's small FP64 kernel before this rule is asked.
+bool pairsum_sym_applies(int64_t nk, bool fp64) { return nk > (fp64 ? 128 : 10752); }
 
 size_t pairsum_sym_work(int64_t nk_pad, int mode, bool fp64, int n_sm, size_t col_budget, int* n_launch) {
     SymPlan p{};

@@ -27,7 +27,7 @@ def kernel_nodes(graph) -> int:
 
 
 CALLS = {}
-for _n, _p in ((500, FP64), (5000, FP64), (3000, TF32), (9000, TF32)):
+for _n, _p in ((500, FP64), (5000, FP64), (3000, TF32), (11000, TF32)):
     CALLS[f"energy_{_n}_{_p}"] = (_n, lambda s, p=_p: vv10.vv10_energy_potential(s.h, p, s.a, s.b, None, False))
 for _n, _P, _p in ((500, 3, FP64), (3000, 3, FP64_TC), (1000, 3, FP64_TC), (3000, 70, FP64_TC), (9000, 54, TF32),
                    (9000, 100, TF32), (3000, 54, F16), (3000, 200, F16)):

@@ -34,7 +34,7 @@ def rows(eng, prec, on):
     vv10.vv10_set_tiles(eng.h, 3 * (prec == FP64), (1 if prec == FP64 else 2) if on else 0, 0)
 
 
-@pytest.mark.parametrize("prec,n", [(MIXED, 9000), (FP64, 5000)], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("prec,n", [(MIXED, 11000), (FP64, 5000)], ids=["mixed", "fp64"])
 def test_no_scratch_at_all(dev, prec, n):
     eng = engine(synth.random_points(n, seed=n), dev)
     try:
@@ -69,7 +69,7 @@ def test_scratch_for_fewer_offsets(dev):
         eng.close()
 
 
-@pytest.mark.parametrize("prec,n", [(MIXED, 9000), (FP64, 5000)], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("prec,n", [(MIXED, 11000), (FP64, 5000)], ids=["mixed", "fp64"])
 def test_captured_without_scratch(dev, prec, n):
     """A call that never ran outside the capture but for the row kernel's buffers."""
     g = synth.random_points(n, seed=n)
