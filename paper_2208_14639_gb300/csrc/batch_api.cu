@@ -304,7 +304,7 @@ vv10_status vv10_ctx::batch_hess(vv10_precision prec, const int32_t* Pt, const d
         for (size_t m = 0; m < n_mol; ++m) {
             const BatchMol& M = B.mol[m];
             if (M.nk == 0) continue;
-            cfg[m].trials_per_cta = hess_f64_trials_per_cta(M.n_t);
+            cfg[m].trials_per_cta = hess_f64_trials_per_cta(M.P, M.n_t, n_sm);
             cfg[m].n_split = hess_f64_default_split(M.P, M.n_t, cfg[m].trials_per_cta, n_sm);
             tpad = std::max(tpad, sizeof(double) * static_cast<size_t>(M.n_t) * M.nk_pad);
             tk = std::max(tk, sizeof(double) * static_cast<size_t>(M.n_t) * M.nk);

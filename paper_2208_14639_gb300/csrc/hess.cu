@@ -207,16 +207,6 @@ static inline void hess_split_geometry(int64_t nk_pad, int req, int64_t& jps, in
     ns = static_cast<int>(ntile > 0 ? cdiv64(ntile, tps) : 1);
 }
 
-// Trials per CTA: the chunks of at most 40 trials (80 FP64 accumulators a thread; eight warps an SM keep
-// the FP64 pipe busy, so registers are there) that need the fewest operations a pair, 31 + 4 per trial
-// and chunk, in the fewest multiples of 4 (1 and 2 for single directions).  Chunks of 8, 16 or 32 did
-// 64 operations for 12 trials' 48.
-int hess_f64_trials_per_cta(int32_t P) {
-    if (P <= 2) return P < 2 ? 1 : 2;
-    const int32_t chunks = static_cast<int32_t>(cdiv64(P, kHessMaxTrials));
-    return static_cast<int>(cdiv64(cdiv64(P, chunks), 4) * 4);
-}
-
 // j splits: between three CTAs an SM and the bound of the partials (six with up to 16 trials), the
 // number that leaves the least work on the fullest SM.
 int hess_f64_default_split(const PointsDev& p, int32_t P, int pc, int n_sm) {
@@ -236,6 +226,31 @@ int hess_f64_default_split(const PointsDev& p, int32_t P, int pc, int n_sm) {
             best = ns;
         }
         if (req > p.nk_pad / kJTile) break;
+    }
+    return best;
+}
+
+// Trials per CTA: the chunks of at most 40 trials (80 FP64 accumulators a thread; eight warps an SM keep
+// the FP64 pipe busy, so registers are there) that need the fewest operations a pair, 31 + 4 per trial
+// and chunk, in the fewest multiples of 4 (1 and 2 for single directions).  Chunks of 8, 16 or 32 did
+// 64 operations for 12 trials' 48.  Where those make less than two CTAs an SM, the width with the fewest
+// operations on the fullest SM: a small system's CTAs take fewer trials each, so that more SMs have one (1,000
+// points, 33 trials: one chunk of 36 1.66 ms, three of 12 0.78; 300 points 1.65 and 0.41).
+int hess_f64_trials_per_cta(const PointsDev& p, int32_t P, int n_sm) {
+    const int64_t rows = cdiv64(p.nk, kHessThreads);
+    const int64_t chunks = cdiv64(P, kHessMaxTrials);
+    int best = P <= 2 ? static_cast<int>(P) : static_cast<int>(cdiv64(cdiv64(P, chunks), 4) * 4);
+    if (rows * chunks * hess_f64_default_split(p, P, best, n_sm) >= 2 * static_cast<int64_t>(n_sm)) return best;
+    int64_t best_ops = -1;
+    for (int pc = best; pc >= 1; pc = pc > 4 ? pc - 4 : pc / 2) {
+        int64_t jps;
+        int ns;
+        hess_split_geometry(p.nk_pad, hess_f64_default_split(p, P, pc, n_sm), jps, ns);
+        const int64_t ops = cdiv64(rows * cdiv64(P, pc) * ns, n_sm) * jps * (31 + 4 * pc);
+        if (best_ops < 0 || ops < best_ops) {
+            best_ops = ops;
+            best = pc;
+        }
     }
     return best;
 }

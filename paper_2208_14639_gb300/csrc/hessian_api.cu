@@ -108,7 +108,7 @@ vv10_status vv10_ctx::hessian(vv10_precision prec, int32_t Pn, const double* rho
         return VV10_OK;
     }
     HessLaunch cfg;
-    cfg.trials_per_cta = hess_f64_trials_per_cta(Pn);
+    cfg.trials_per_cta = hess_f64_trials_per_cta(P, Pn, n_sm);
     cfg.n_split = hess_f64_default_split(P, Pn, cfg.trials_per_cta, n_sm);
     H_TRY(ensure(hacc, sizeof(double) * 2 * static_cast<size_t>(cfg.n_split) * Pn * P.nk_pad,
                  "contraction partials"));

@@ -339,7 +339,7 @@ struct HessLaunch {
     int n_split = 1;
 };
 int hess_f64_default_split(const PointsDev& p, int32_t P, int pc, int n_sm);
-int hess_f64_trials_per_cta(int32_t P);
+int hess_f64_trials_per_cta(const PointsDev& p, int32_t P, int n_sm);
 // acc: [2][n_split][P][nk_pad] partial sums of the pair part (rho row, gamma row).
 cudaError_t launch_hess_f64(const PointsDev& p, int32_t P, const double* u, const double* y,
                             const HessLaunch& cfg, double* acc, int* err, cudaStream_t st);
