@@ -77,8 +77,9 @@ k_ao_z(PointsDev P, int32_t nbf, int32_t nc, bool weight, const double* __restri
     const double w = weight ? P.w[k] : 1.0;
     const AoCoef* cf = coef + k * nc;
     double* z = Z + k * nc * nbf + mu;
+    const int per = (nc + gridDim.y - 1) / gridDim.y, c1 = min(nc, static_cast<int>(blockIdx.y + 1) * per);
 #pragma unroll 4
-    for (int c = 0; c < nc; ++c) {
+    for (int c = blockIdx.y * per; c < c1; ++c) {
         const AoCoef t = cf[c];
         z[static_cast<int64_t>(c) * nbf] = w * fma(t.a, f, fma(t.z, dz, fma(t.y, dy, t.x * dx)));
     }
@@ -227,8 +228,11 @@ cudaError_t assemble_chunks(const PointsDev& p, const AoGemm& g, int32_t nbf, in
         make_coef(c0, nc, coef);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_ao_z<<<static_cast<unsigned>((p.nk * nbf + 255) / 256), 256, 0, st>>>(p, nbf, nc, weight, phi, dphi,
-                                                                                coef, Z);
+        // few points and functions: the channels over several CTAs, so that the chip has two a SM
+        const int64_t gx = (p.nk * nbf + 255) / 256;
+        const int64_t gy = gx >= 2 * g.n_sm ? 1 : (2 * g.n_sm / gx < nc ? 2 * g.n_sm / gx : nc);
+        k_ao_z<<<dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy)), 256, 0, st>>>(p, nbf, nc, weight, phi,
+                                                                                         dphi, coef, Z);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         // one product for the chunk: M (column-major nbf x nc nbf) = A B^T with A = phik
