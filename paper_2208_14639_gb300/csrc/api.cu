@@ -1007,7 +1007,7 @@ static vv10_status ao_assemble(vv10_handle h, int32_t nbf, const double* phi, co
     VV10_TRY(h->ensure(h->aoz, sizeof(double) * (nk * (nbf + 4) * chunk + 1), "assembly operand"));
     VV10_TRY(h->ensure(h->aom, sizeof(double) * static_cast<size_t>(nbf) * nbf * chunk, "assembly products"));
     const size_t gw = ao_gemm_work_elems(nbf, chunk, h->n_sm);
-    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), P.nk), "assembly product partials"));
+    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf, nbf * chunk, P.nk, h->n_sm), "assembly product partials"));
     int launched = 0;
     const AoGemm g{static_cast<double*>(h->aogw.p), gw, reinterpret_cast<int32_t*>(static_cast<double*>(h->aogw.p) + gw),
                    h->n_sm, &launched, static_cast<int*>(h->dev_err.p)};
@@ -1093,7 +1093,7 @@ vv10_status vv10_fock_derivative(vv10_handle h, int32_t nbf, const double* phi,
     VV10_TRY(h->ensure(h->aom, sizeof(double) * nn * chunk, "assembly products"));
     VV10_TRY(h->ensure(h->aofa, sizeof(double) * (4 * nk * nbf + 2 * nn), "basis-derivative factors"));
     const size_t gw = ao_gemm_work_elems(nbf, chunk, h->n_sm);
-    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf * (chunk + 1), P.nk), "assembly product partials"));
+    VV10_TRY(h->ensure(h->aogw, sizeof(double) * gw + sizeof(int32_t) * gemm_slices_expo_ints(nbf, nbf * chunk, P.nk, h->n_sm), "assembly product partials"));
     int launched = 0;
     const AoGemm g{static_cast<double*>(h->aogw.p), gw, reinterpret_cast<int32_t*>(static_cast<double*>(h->aogw.p) + gw),
                    h->n_sm, &launched, static_cast<int*>(h->dev_err.p)};

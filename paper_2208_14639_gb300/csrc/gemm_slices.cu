@@ -69,7 +69,7 @@ struct GsArgs {
     const double *A, *B;
     int64_t lda, ldb;
     const int32_t *ea, *eb;      // [block][row] biased exponent of the row's largest |element|, or kGsPlain
-    const int32_t* plain;        // not 0: some row's block is kGsPlain
+    int32_t* plain;              // [split][tile of C]: whether a row of its block range is kGsPlain
     double* part;                // [split][N][M]
     int* err;
 };
@@ -89,8 +89,9 @@ __device__ __forceinline__ bool gs_wait(uint64_t* bar, uint32_t parity, int* err
 }
 
 // Rows `row0 + (lane & 7)` of a tile (8 rows of this warp) x a stage's 32 k: slices into smem (slice p
-// at base + p slice_bytes).  X: element (row, k) at k ld + row; emax: the block's exponents.
-__device__ __forceinline__ void gs_cut(const double* __restrict__ X, int64_t ld, int rows, int first,
+// at base + p slice_bytes).  X: element (row, k) at k ld + row; emax: the block's exponents.  Returns
+// whether this lane's row is kGsPlain.
+__device__ __forceinline__ bool gs_cut(const double* __restrict__ X, int64_t ld, int rows, int first,
                                        int row0, int64_t k0, int64_t K, const int32_t* __restrict__ emax,
                                        uint8_t* base, uint32_t slice_bytes) {
     const int lane = threadIdx.x & 31;
@@ -132,6 +133,7 @@ __device__ __forceinline__ void gs_cut(const double* __restrict__ X, int64_t ld,
         }
         tc::st_shared_v4(at + p * slice_bytes, w[0], w[1], w[2], w[3]);
     }
+    return !real && first + r < rows;
 }
 
 __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
     uint64_t* acc_free = bars + 4;   // the accumulators of a block are read
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 6);
+    volatile int* plain_flag = abort_flag + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         mbar_init(&full[0], kGsWarps);
@@ -152,6 +155,7 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
         mbar_init(&mma_done[1], 1);
         mbar_init(acc_free, kGsWarps);
         *abort_flag = 0;
+        *plain_flag = 0;
         fence_mbar_init();
     }
     if (warp == kGsWarps) tc::tmem_alloc(tmem_slot, 512);
@@ -208,7 +212,7 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
             if (lane == 0) mbar_arrive(acc_free);
             return true;
         };
-        bool ok = true;
+        bool ok = true, plain = false;
         for (int s = 0; s < ns && ok; ++s) {
             const int64_t blk = b0 + s / kGsBlk;
             if (s >= 2) {  // the buffer is free once the MMAs of stage s - 2 are done
@@ -222,14 +226,15 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
             const int64_t k0 = (blk * kGsBlk + s % kGsBlk) * kGsK;
             for (int r0 = 8 * warp; r0 < kGsM; r0 += 8 * kGsWarps)
                 if (m0 + r0 < args.M || s < 2)  // rows past M: zeros, once per buffer
-                    gs_cut(args.A, args.lda, args.M, m0, r0, k0, args.K, args.ea + blk * args.M, buf, kGsABytes);
-            gs_cut(args.B, args.ldb, args.N, n0, 8 * warp, k0, args.K, args.eb + blk * args.N,
-                   buf + kGsSlices * kGsABytes, kGsBBytes);
+                    plain |= gs_cut(args.A, args.lda, args.M, m0, r0, k0, args.K, args.ea + blk * args.M, buf, kGsABytes);
+            plain |= gs_cut(args.B, args.ldb, args.N, n0, 8 * warp, k0, args.K, args.eb + blk * args.N,
+                            buf + kGsSlices * kGsABytes, kGsBBytes);
             tc::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[s & 1]);
             if (s > 0 && s % kGsBlk == 0) ok = combine(s / kGsBlk - 1);
         }
+        if (plain) *plain_flag = 1;  // every writer the same value
         if (ok && combine(ns / kGsBlk - 1) && m < args.M) {
             double* out = args.part + static_cast<int64_t>(blockIdx.z) * args.M * args.N + m;
 #pragma unroll
@@ -264,6 +269,8 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
     }
     tc::fence_before();
     __syncthreads();
+    if (threadIdx.x == 0)
+        args.plain[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = *plain_flag;
     if (warp == kGsWarps) {
         tc::fence_after();
         tc::tmem_dealloc(tmem, 512);
@@ -272,7 +279,7 @@ __global__ void __launch_bounds__(kGsThreads, 1) k_gemm_slices(GsArgs args) {
 
 // emax[block][row] = biased exponent of the row's largest |element| in the block's 128 k, or kGsPlain.
 __global__ void __launch_bounds__(256) k_exp_max(const double* __restrict__ X, int64_t ld, int rows, int64_t K,
-                                                 int32_t* __restrict__ emax, int32_t* __restrict__ plain) {
+                                                 int32_t* __restrict__ emax) {
     __shared__ int sh[4][64];
     const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
     const int r = blockIdx.y * 64 + c;
@@ -286,11 +293,7 @@ __global__ void __launch_bounds__(256) k_exp_max(const double* __restrict__ X, i
     __syncthreads();
     if (g == 0 && r < rows) {
         e = max(max(sh[0][c], sh[1][c]), max(sh[2][c], sh[3][c]));
-        if (e > kGsBig) {
-            e = kGsPlain;
-            *plain = 1;  // every writer the same value
-        }
-        emax[static_cast<int64_t>(blockIdx.x) * rows + r] = e;
+        emax[static_cast<int64_t>(blockIdx.x) * rows + r] = e > kGsBig ? kGsPlain : e;
     }
 }
 
@@ -300,9 +303,15 @@ __global__ void k_slices_reduce(GsArgs a, int n_split, double* __restrict__ C, i
     const int64_t mn = static_cast<int64_t>(a.M) * a.N;
     if (e >= mn) return;
     const int64_t n = e / a.M, m = e % a.M;
+    const int tiles_m = (a.M + kGsM - 1) / kGsM, tiles = tiles_m * ((a.N + kGsN - 1) / kGsN);
+    const int32_t* plain = a.plain + n / kGsN * tiles_m + m / kGsM;
     double s = 0.0;
-    for (int z = 0; z < n_split; ++z) s += a.part[z * mn + e];
-    if (*a.plain)
+    int any = 0;
+    for (int z = 0; z < n_split; ++z) {
+        s += a.part[z * mn + e];
+        any |= plain[z * tiles];
+    }
+    if (any)
         for (int64_t b = 0; b < a.n_blk; ++b) {
             if (a.ea[b * a.M + m] >= 0 && a.eb[b * a.N + n] >= 0) continue;
             const int64_t k1 = min(a.K, (b + 1) * kGsBlk * kGsK);
@@ -313,8 +322,10 @@ __global__ void k_slices_reduce(GsArgs a, int n_split, double* __restrict__ C, i
 
 }  // namespace
 
-size_t gemm_slices_expo_ints(int64_t rows, int64_t K) {  // the rows' exponents and the flag `plain`
-    return static_cast<size_t>(rows) * static_cast<size_t>((K + kGsBlk * kGsK - 1) / (kGsBlk * kGsK)) + 1;
+// The rows' exponents, and `plain` of at most max(tiles of C, 8 n_sm) CTAs (gemm_slices_splits).
+size_t gemm_slices_expo_ints(int64_t M, int64_t N, int64_t K, int n_sm) {
+    const int64_t tiles = ((M + kGsM - 1) / kGsM) * ((N + kGsN - 1) / kGsN), cap = 8 * static_cast<int64_t>(n_sm);
+    return static_cast<size_t>((M + N) * ((K + kGsBlk * kGsK - 1) / (kGsBlk * kGsK)) + (tiles > cap ? tiles : cap));
 }
 
 // From 512 k: four blocks and the two exponent passes cost less than the FMA kernel's steps at every M
@@ -362,13 +373,10 @@ cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t
     a.err = err;
     const unsigned nb = static_cast<unsigned>(a.n_blk);
     int32_t* expo_b = expo + static_cast<int64_t>(nb) * M;
-    int32_t* plain = expo_b + static_cast<int64_t>(nb) * N;
-    a.plain = plain;
+    a.plain = expo_b + static_cast<int64_t>(nb) * N;
     *launched += 4;
-    e = cudaMemsetAsync(plain, 0, sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
-    k_exp_max<<<dim3(nb, static_cast<unsigned>((M + 63) / 64)), 256, 0, st>>>(A, lda, M, K, expo, plain);
-    k_exp_max<<<dim3(nb, static_cast<unsigned>((N + 63) / 64)), 256, 0, st>>>(B, ldb, N, K, expo_b, plain);
+    k_exp_max<<<dim3(nb, static_cast<unsigned>((M + 63) / 64)), 256, 0, st>>>(A, lda, M, K, expo);
+    k_exp_max<<<dim3(nb, static_cast<unsigned>((N + 63) / 64)), 256, 0, st>>>(B, ldb, N, K, expo_b);
     const dim3 grid(static_cast<unsigned>((M + kGsM - 1) / kGsM), static_cast<unsigned>((N + kGsN - 1) / kGsN),
                     static_cast<unsigned>(n_split));
     k_gemm_slices<<<grid, kGsThreads, kGsSmem, st>>>(a);

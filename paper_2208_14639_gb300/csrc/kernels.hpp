@@ -418,9 +418,9 @@ cudaError_t launch_gemm_abt(int M, int N, int64_t K, const double* A, int64_t ld
                             int* launched, cudaStream_t st);
 
 // The same product on the tensor cores, as exact integer slice products (gemm_slices.cu); work as
-// above, expo: gemm_slices_expo_ints(M + N, K), err: the device error word.
+// above, expo: gemm_slices_expo_ints, err: the device error word.
 // gemm_slices_applies: where it is faster.
-size_t gemm_slices_expo_ints(int64_t rows, int64_t K);
+size_t gemm_slices_expo_ints(int64_t M, int64_t N, int64_t K, int n_sm);
 bool gemm_slices_applies(int64_t K);
 int gemm_slices_splits(int M, int N, int64_t K, int n_sm, size_t work_elems);
 cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t lda, const double* B,
@@ -431,7 +431,7 @@ cudaError_t launch_gemm_slices(int M, int N, int64_t K, const double* A, int64_t
 // M_c + M_c^T, M_c = Phi^T Z_c over the kept points, channels in chunks of `chunk`
 // (ao_channels_per_chunk).  Scratch: phik (nk x nbf), Z and its coefficients (chunk x nk x (nbf +
 // 4), + 1), M (chunk x nbf x nbf) and the product's split-K partials (AoGemm: ao_gemm_work_elems
-// doubles, and the exponents of a product of (chunk + 1) nbf rows over nk points).
+// doubles, and gemm_slices_expo_ints of nbf x chunk nbf over nk points).
 struct AoGemm {
     double* work;
     size_t work_elems;
