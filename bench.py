@@ -78,7 +78,7 @@ PROFILED_TRAFFIC = {
     # k_hess_f16 on the 60-atom grid (P = 180, one 192-wide group, 24 MB j chunks, evict-last
     # trial tiles, streaming partial output): ncu dram__bytes_read.sum + dram__bytes_write.sum
     # of one launch
-    ("k_hess_f16", "chon60"): 630.09e9 + 194.94e9,
+    ("k_hess_f16", "chon60"): 1.94e12 + 197.83e9,
 }
 
 

@@ -451,7 +451,10 @@ vv10_status vv10_sync(vv10_handle h, void* stream);
 /* Tile shapes (the paper has no counterpart).  `what` selects a kernel:
  *   0..5  single-system pair sums, mode + 3 * fp64 (mode 0 = energy/potential sums, 1 = the
  *         A/B/C sums of the Hessian diagonal, 2 = coordinate gradient): rows_per_thread in
- *         {1, 2, 4} (FP64: {1, 2}), n_split = number of j-splits (0 = from the SM count);
+ *         {1, 2, 4} (FP64: {1, 2}), n_split = number of j-splits (0 = from the SM count).
+ *         These are shapes of the row-by-row kernel: fixing one makes it run at every size
+ *         (by itself it runs in the mixed modes up to 10,752 kept points, and where the
+ *         other kernels' scratch is not to be had);
  *   6, 7  batched pair sums, 6 + fp64: rows_per_thread as above, n_split = j tiles (of 256
  *         points) per split (0 = 32);
  *   8     tensor-core contraction: rows_per_thread = the widest trial group, in [32, 192];
@@ -498,7 +501,8 @@ vv10_status vv10_set_options(vv10_handle h, int flags);
 /* Autotuner (the paper has no counterpart).  Times every candidate shape of a kernel (see
  * vv10_set_tiles) on the handle's prepared data, on `stream`, and applies the fastest:
  *   VV10_TUNE_PAIRSUMS     the three pair-sum modes of the prepared single system (for prec:
- *                          rows per thread x {default, half, twice} the j-splits);
+ *                          rows per thread x {default, half, twice} the j-splits), where the
+ *                          row-by-row kernel runs;
  *   VV10_TUNE_BATCH        the batched pair sums of the prepared batch (for prec: rows per
  *                          thread x {16, 32, 64} j tiles per split);
  *   VV10_TUNE_CONTRACTION  the widest trial group of the mixed contraction (64, 96, 128,
