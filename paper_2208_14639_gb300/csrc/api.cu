@@ -501,6 +501,8 @@ TileChoice vv10_ctx::tiles_for(int mode, bool fp64) const {
     if (use) {
         t.rows_per_thread = use->rows_per_thread;
         t.n_split = use->n_split;
+        if (!use->manual && use->bucket < 0)  // not timed: the default of the present size
+            t.n_split = pairsum_default_split(P, mode, fp64, t.rows_per_thread, n_sm);
     }
     return t;
 }

@@ -129,9 +129,10 @@ vv10_status vv10_ctx::tune_pairsum(int mode, bool fp64, cudaStream_t st, bool fo
     }
     float best = 3.0e38f;
     int best_r = fp64 ? 1 : 2, best_s = 0;
-    // no shape to choose where the unordered-pair or the small FP64 kernel runs
+    // no shape to choose where the unordered-pair or the small FP64 kernel runs: the default one, for no
+    // bucket (a size of the row kernel in this bucket is still to be timed)
     if (pairsum_sym(mode, fp64) || (fp64 && pairsum_rows64_applies(P.nk))) {
-        o = TileOverride{true, false, mode, fp64, best_r, pairsum_default_split(P, mode, fp64, best_r, n_sm), nb};
+        o = TileOverride{true, false, mode, fp64, best_r, 0, -1};
         return VV10_OK;
     }
     if (stream_capturing(st)) return VV10_OK;
