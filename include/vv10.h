@@ -87,9 +87,9 @@ typedef struct vv10_ctx* vv10_handle;
 #define VV10_MAX_BASIS 4096
 
 /* Create a handle bound to CUDA device `device`.  Allocates no large buffers yet: a call allocates the
- * scratch that it lacks, and a buffer grows when a call needs more of it.  So make a call once before it is
- * captured, and capture it again after a call with more points, trials or sums, or in another
- * precision of the pair sums: a smaller one in the same precision leaves every buffer in place.
+ * scratch that it lacks, and a buffer moves when a call needs more of it.  So make a call once before it is
+ * captured, and capture it again when calls in between may have needed more: more points, trials or sums,
+ * another precision; the FP64 contraction's partials can grow with fewer trials too.
  * Errors: INVALID_ARG (h NULL, bad device), CUDA. */
 vv10_status vv10_create(vv10_handle* h, int device);
 
